@@ -123,6 +123,19 @@ const char* hf_strerror(int status)
 
 const char* hf_last_error(void) { return g_err.c_str(); }
 
+static void ctx_release(hf_ctx* c)
+{
+    DeviceGuard g(c->device);
+    for (auto& ev : c->ev)
+        if (ev) cudaEventDestroy(ev);
+    for (int i = 0; i < kSideStreams; i++) {
+        if (c->join[i]) cudaEventDestroy(c->join[i]);
+        if (c->side[i]) cudaStreamDestroy(c->side[i]);
+    }
+    if (c->fork) cudaEventDestroy(c->fork);
+    delete c;
+}
+
 int hf_create(hf_ctx** out, int device, void* cuda_stream)
 {
     if (!out) return fail(HF_E_INVALID, "hf_create: ctx pointer is NULL");
@@ -175,23 +188,19 @@ int hf_create(hf_ctx** out, int device, void* cuda_stream)
                 break;
             }
         }
-        c->events_ready = (rc == HF_OK);
+        for (int i = 0; i < kSideStreams && rc == HF_OK; i++)
+            if (cudaStreamCreateWithFlags(&c->side[i], cudaStreamNonBlocking) != cudaSuccess ||
+                cudaEventCreateWithFlags(&c->join[i], cudaEventDisableTiming) != cudaSuccess)
+                rc = cuda_status(cudaGetLastError(), "hf_create: side stream");
+        if (rc == HF_OK && cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) != cudaSuccess)
+            rc = cuda_status(cudaGetLastError(), "cudaEventCreate");
     }
     if (rc != HF_OK) {
-        delete c;
+        ctx_release(c);
         return rc;
     }
     *out = c;
     return HF_OK;
-}
-
-static void ctx_release(hf_ctx* c)
-{
-    DeviceGuard g(c->device);
-    if (c->events_ready)
-        for (auto& ev : c->ev)
-            if (ev) cudaEventDestroy(ev);
-    delete c;
 }
 
 void hf_destroy(hf_ctx* c)
@@ -704,12 +713,24 @@ static bool uses_rys(int ci, int flags, int use_f32, const EriArgs& a)
 }
 // (the ket tables always exist for a class with significant pairs, so a.kt is set for every launch)
 
+// One class launch of a build.
+struct ClassLaunch {
+    int ci, prec, use_f32, lanes, grid;
+    double est;  // estimated device time, in operations of the whole GPU
+};
+
 // The per-class ERI launches shared by hf_fock_build, hf_fock_build_partial and hf_fock_build_noalloc.
+//
+// Small systems: a class with a few hundred quartets lasts as long as its slowest quartet whatever the GPU
+// could do beside it, and the classes' launches, one after another, add those latencies up (one water: 21
+// launches of 0.1 to 5.8 ms each for 0.05 ms of arithmetic).  The launches are independent (they only add
+// into J and K), so they are spread over the side streams, the longest first (by the larger of the class's
+// share of the GPU's rate and the latency of one quartet), each to the stream with the least work so far.
+// Large systems gain the same way at each class's tail.
 int hf::launch_eri_classes(hf_system* S, EriArgs a, int shard, int n_shards, int flags, cudaEvent_t* ev,
                            unsigned long long* prim_count)
 {
     hf_ctx* ctx = S->ctx;
-    cudaStream_t st = ctx->stream;
     hf_system& X = *S;
     a.pairs = S->pairs.as<PairHdr>();
     a.prims64 = S->prims64.p;
@@ -718,57 +739,86 @@ int hf::launch_eri_classes(hf_system* S, EriArgs a, int shard, int n_shards, int
     a.boys64 = ctx->boys64.as<double>();
     a.boys32 = ctx->boys32.as<float>();
     a.prim_tau = S->th.prim_tau;
-    for (int ci = 0; ci < kNumClasses; ci++) {
-        const auto& pl = S->plan[ci];
-        const int Xc = kEriClasses[ci].X, Yc = kEriClasses[ci].Y;
+    ClassLaunch todo[2 * kNumClasses];
+    int n_todo = 0;
+    for (int ci = 0; ci < kNumClasses; ci++)
+        for (int prec = 0; prec < 2; prec++) {
+            const long long n = prec ? S->plan[ci].n32 : S->plan[ci].n64;
+            const long long nq = n * (shard + 1) / n_shards - n * shard / n_shards;
+            ClassLaunch c{ci, prec, prec && !(flags & HF_FP64_ONLY), 1, 0, 0.0};
+            // a class too small to fill the GPU with one thread per quartet shares each quartet's
+            // primitive work among a lane group instead (shorter latency, same result)
+            if (!c.use_f32 && nq < (long long)ctx->num_sms * 256) c.lanes = kEriClasses[ci].lanes;
+            const long long blocks = (nq * c.lanes + kEriThreads - 1) / kEriThreads;
+            c.grid = (int)std::min<long long>(blocks, (long long)ctx->num_sms * 16);
+            // one quartet's operations run in one lane group, 1 / (64 lanes SMs) of the GPU at a time
+            const double ops = (double)kEriClasses[ci].prim_flops * X.maxpp * X.maxpp / c.lanes + kEriClasses[ci].cont_flops;
+            c.est = std::max((double)nq * c.lanes, 64.0 * ctx->num_sms) * ops / (c.use_f32 ? 32.0 : 1.0);
+            if (nq > 0 || ev) todo[n_todo++] = c;
+        }
+    const bool forked = !ev && n_todo > 1;
+    double load[kSideStreams] = {};
+    if (forked) {
+        std::sort(todo, todo + n_todo, [](const ClassLaunch& x, const ClassLaunch& y) { return x.est > y.est; });
+        HF_CUDA(cudaEventRecord(ctx->fork, ctx->stream));
+        for (int i = 0; i < std::min(kSideStreams, n_todo); i++) HF_CUDA(cudaStreamWaitEvent(ctx->side[i], ctx->fork, 0));
+    }
+    cudaError_t err = cudaSuccess;
+    for (int t = 0; t < n_todo && err == cudaSuccess; t++) {
+        const ClassLaunch& c = todo[t];
+        const auto& pl = S->plan[c.ci];
+        const int Xc = kEriClasses[c.ci].X, Yc = kEriClasses[c.ci].Y;
+        cudaStream_t st = ctx->stream;
+        if (forked) {
+            const int i = (int)(std::min_element(load, load + kSideStreams) - load);
+            load[i] += c.est;
+            st = ctx->side[i];
+        }
         a.bra = S->class_ids[Xc].as<int>();
         a.ket = S->class_ids[Yc].as<int>();
         a.bhdr = S->class_hdr[Xc].as<PairHdr>();
         a.khdr = S->class_hdr[Yc].as<PairHdr>();
         a.n_bra = S->class_count[Xc];
         a.same = Xc == Yc;
-        for (int prec = 0; prec < 2; prec++) {
-            const long long n = prec ? pl.n32 : pl.n64;
-            const long long q0 = n * shard / n_shards, q1 = n * (shard + 1) / n_shards;
-            if (ev) HF_CUDA(cudaEventRecord(ev[4 * ci + 2 * prec], st));
-            a.prim_count = prim_count ? prim_count + 2 * ci + prec : nullptr;
-            if (q1 > q0) {
-                a.offsets = prec ? pl.offsets32.as<long long>() : pl.offsets64.as<long long>();
-                a.kstart = prec ? pl.kstart32.as<int>() : nullptr;
-                a.chunk = prec ? pl.chunk32.as<int>() : pl.chunk64.as<int>();
-                a.q_begin = q0;
-                a.n_quartets = q1;
-                const int use_f32 = prec && !(flags & HF_FP64_ONLY);
-                a.kt = nullptr;
-                a.ktB = nullptr;
-                a.kstride = 0;
-                if (X.ket_tab[Yc].p) {
-                    const long long st_ = X.ket_stride[Yc];
-                    const double* t64 = X.ket_tab[Yc].as<double>();
-                    const float* t32 = (const float*)(t64 + 9 * (size_t)X.maxpp * st_);
-                    a.kt = use_f32 ? (const void*)t32 : (const void*)t64;
-                    a.ktB = t32 + 9 * (size_t)X.maxpp * st_;
-                    a.kstride = st_;
-                }
-                // a class too small to fill the GPU with one thread per quartet shares each quartet's
-                // primitive work among a lane group instead (shorter latency, same result)
-                const int lanes = (!use_f32 && q1 - q0 < (long long)ctx->num_sms * 256) ? kEriClasses[ci].lanes : 1;
-                const long long blocks = ((q1 - q0) * lanes + kEriThreads - 1) / kEriThreads;
-                const int grid = (int)std::min<long long>(blocks, (long long)ctx->num_sms * 16);
-                // FP64 launches run each warp's window of quartets sorted by staircase length (64 waters:
-                // 2% faster); the FP32 kernels, bound by latency rather than a pipe, ran 10% slower with it
-                // and are compiled without it
-                a.sort_work = use_f32 ? 0 : 1;
-                if (uses_rys(ci, flags, use_f32, a))
-                    kEriClasses[ci].launch_rys(a, 0, grid, kEriThreads, st, lanes);
-                else
-                    kEriClasses[ci].launch(a, use_f32, grid, kEriThreads, st, lanes);
-                HF_CUDA(cudaGetLastError());
+        const long long n = c.prec ? pl.n32 : pl.n64;
+        a.q_begin = n * shard / n_shards;
+        a.n_quartets = n * (shard + 1) / n_shards;
+        if (ev) err = cudaEventRecord(ev[4 * c.ci + 2 * c.prec], st);
+        a.prim_count = prim_count ? prim_count + 2 * c.ci + c.prec : nullptr;
+        if (a.n_quartets > a.q_begin && err == cudaSuccess) {
+            a.offsets = c.prec ? pl.offsets32.as<long long>() : pl.offsets64.as<long long>();
+            a.kstart = c.prec ? pl.kstart32.as<int>() : nullptr;
+            a.chunk = c.prec ? pl.chunk32.as<int>() : pl.chunk64.as<int>();
+            a.kt = nullptr;
+            a.ktB = nullptr;
+            a.kstride = 0;
+            if (X.ket_tab[Yc].p) {
+                const long long st_ = X.ket_stride[Yc];
+                const double* t64 = X.ket_tab[Yc].as<double>();
+                const float* t32 = (const float*)(t64 + 9 * (size_t)X.maxpp * st_);
+                a.kt = c.use_f32 ? (const void*)t32 : (const void*)t64;
+                a.ktB = t32 + 9 * (size_t)X.maxpp * st_;
+                a.kstride = st_;
             }
-            if (ev) HF_CUDA(cudaEventRecord(ev[4 * ci + 2 * prec + 1], st));
+            // FP64 launches run each warp's window of quartets sorted by staircase length (64 waters:
+            // 2% faster); the FP32 kernels, bound by latency rather than a pipe, ran 10% slower with it
+            // and are compiled without it
+            a.sort_work = c.use_f32 ? 0 : 1;
+            if (uses_rys(c.ci, flags, c.use_f32, a))
+                kEriClasses[c.ci].launch_rys(a, 0, c.grid, kEriThreads, st, c.lanes);
+            else
+                kEriClasses[c.ci].launch(a, c.use_f32, c.grid, kEriThreads, st, c.lanes);
+            err = cudaGetLastError();
         }
+        if (ev && err == cudaSuccess) err = cudaEventRecord(ev[4 * c.ci + 2 * c.prec + 1], st);
     }
-    return HF_OK;
+    if (forked)  // joined whether or not a launch failed: what was launched still uses the system's buffers
+        for (int i = 0; i < std::min(kSideStreams, n_todo); i++) {
+            const cudaError_t e1 = cudaEventRecord(ctx->join[i], ctx->side[i]);
+            const cudaError_t e2 = cudaStreamWaitEvent(ctx->stream, ctx->join[i], 0);
+            if (err == cudaSuccess) err = e1 != cudaSuccess ? e1 : e2;
+        }
+    return err == cudaSuccess ? HF_OK : cuda_status(err, "ERI class launch");
 }
 
 extern "C" {

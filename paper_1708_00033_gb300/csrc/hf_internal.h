@@ -16,6 +16,7 @@ constexpr int kNumPairClasses = 6;  // ss ps pp ds dp dd
 constexpr int kNumClasses = 21;     // (X|Y), X >= Y
 constexpr int kChunkShift = 10;      // quartets per entry of the bra lookup tables: 1024
 constexpr int kMaxPrim = 8;         // primitives per shell accepted by the library
+constexpr int kSideStreams = 8;     // streams the class launches of one build are spread over
 
 // One significant shell pair, oriented so that l_A >= l_B.
 struct PairHdr {
@@ -134,6 +135,8 @@ inline bool class_uses_rys(int ci, int flags)
 // [n shard / n_shards, n (shard + 1) / n_shards) of its n screened quartets (shard 0 of 1 is the
 // whole build).  `a` carries the fields common to every launch (density, accumulators, tables,
 // screening and flag pointers); the per-class fields are filled here.  flags: HF_FP64_ONLY.
+// The launches run concurrently on the context's side streams, between an event recorded on the context's
+// stream and one it waits for; with ev they run one after another on the context's stream instead.
 // ev (nullable): events 4 c + 2 prec and 4 c + 2 prec + 1 are recorded around each class launch;
 // prim_count (nullable): 2 c + prec counts the evaluated primitive quartets of each launch.
 int launch_eri_classes(hf_system* S, EriArgs a, int shard, int n_shards, int flags, cudaEvent_t* ev,
@@ -188,9 +191,10 @@ struct hf_ctx {
     int num_sms = 0;
     hf::DevBuf boys64, boys32;  // Boys Taylor tables
     cudaEvent_t ev[4 * hf::kNumClasses + 4] = {};
-    bool events_ready = false;
     int n_systems = 0;            // live systems created on this context
     bool destroy_pending = false;  // hf_destroy was called while systems were alive
+    cudaStream_t side[hf::kSideStreams] = {};  // class launches of one build run on these, forked from and
+    cudaEvent_t fork = nullptr, join[hf::kSideStreams] = {};  // joined to `stream` (launch_eri_classes)
     void* noalloc_scratch = nullptr;  // device address of hf_fock_build_noalloc's fixed scratch
 };
 
