@@ -9,8 +9,8 @@
  * the direct-SCF algorithm of Section 4: the symmetry-unique shell quartets of
  * Algorithm 1, Cauchy-Schwarz screened, each electron-repulsion integral
  * applied to the six Fock elements of Eq. 1a-1f.  Integrals are evaluated on
- * the GPU by Obara-Saika / Head-Gordon-Pople recurrences over contracted
- * Cartesian Gaussians (the paper treats eri() as a black box).
+ * the GPU over contracted Cartesian Gaussians by Hermite (McMurchie-Davidson),
+ * Obara-Saika or Rys kernels (the paper treats eri() as a black box).
  *
  * Conventions (every entry point):
  *   - Units are atomic units (bohr, hartree).
@@ -57,14 +57,14 @@ extern "C" {
                                 largest |P| of the six density blocks they touch (x4) is below schwarz_tau */
 #define HF_RYS 32            /* hf_fock_build, hf_fock_build_partial: evaluate the FP64 quartets of all five
                                 classes of total angular momentum L >= 6 ((dp|dp), (dd|pp), (dd|ds), (dd|dp),
-                                (dd|dd)) by Rys quadrature (L/2 + 1 nodes of the Boys weight) instead of the
-                                Obara-Saika vertical recurrence; the contraction, horizontal recurrence and
-                                digestion are shared, so results agree to rounding.  Without HF_RYS or
-                                HF_OBARA_SAIKA the builds use Rys for the four of them where it is faster
-                                ((dp|dp), (dd|ds), (dd|dp), (dd|dd)) and Obara-Saika for (dd|pp).  FP32
-                                launches and the batched builds always use Obara-Saika. */
-#define HF_OBARA_SAIKA 64    /* hf_fock_build, hf_fock_build_partial: Obara-Saika for every class (no Rys);
-                                with HF_RYS as well, HF_OBARA_SAIKA wins */
+                                (dd|dd)) by Rys quadrature (L/2 + 1 nodes of the Boys weight); the other classes
+                                keep the default method. */
+#define HF_OBARA_SAIKA 64    /* hf_fock_build, hf_fock_build_partial: the Obara-Saika vertical recurrence for the
+                                FP64 quartets of every class; with HF_RYS as well, HF_OBARA_SAIKA wins.
+                                Without either flag FP64 quartets, those of the batched builds and the Schwarz
+                                bounds use McMurchie-Davidson Hermite integrals accumulated over the primitives
+                                before the pair geometry enters;
+                                the results agree to rounding.  FP32 launches always use Obara-Saika. */
 
 typedef struct hf_ctx hf_ctx;       /* one device + one stream + constant tables */
 typedef struct hf_system hf_system; /* one molecule: basis, pairs, screening plan, 1e matrices */

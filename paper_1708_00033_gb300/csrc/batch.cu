@@ -127,6 +127,7 @@ struct hf_batch {
     hf_ctx* ctx = nullptr;
     int device = 0;
     int n_mol = 0;
+    ExponentTable etab;  // shared by the molecules' systems: one table in L2 instead of one per molecule
     std::vector<hf_system*> sys;
     std::vector<long long> eoff_h;  // [n_mol + 1]
     long long len = 0;
@@ -171,6 +172,12 @@ static BatchArgs batch_args(hf_batch* B, int c, long long limit)
     return a;
 }
 
+// persistent grid: bps blocks per SM of the thread kernels, twice as many of the one-warp blocks
+static int batch_grid(const hf_batch* B, int c, int bps)
+{
+    return B->num_sms * bps * (kEriClasses[c].batch_warp ? 2 : 1);
+}
+
 static int capture_graph(hf_batch* B)
 {
     if (B->exec) {
@@ -193,7 +200,7 @@ static int capture_graph(hf_batch* B)
         if (B->n_total[c] <= 0) continue;
         cudaStreamWaitEvent(B->cst[c], B->fork, 0);
         const BatchArgs a = batch_args(B, c, -1);
-        kEriClasses[c].launch_batch(a, B->num_sms * B->bps[c], B->block[c], B->cst[c]);
+        kEriClasses[c].launch_batch(a, batch_grid(B, c, B->bps[c]), B->block[c], B->cst[c]);
         cudaEventRecord(B->join[c], B->cst[c]);
         cudaStreamWaitEvent(st, B->join[c], 0);
     }
@@ -228,8 +235,13 @@ int hf_batch_create(hf_ctx* ctx, int n_mol, const hf_geometry* geoms, const hf_b
     if (th) t = *th;
     t.fp32_cutoff = 0.0;  // the batched path is FP64 throughout
     for (int m = 0; m < n_mol; m++) {
+        if (int rc = check_geometry_basis(&geoms[m], &bases[m], &t)) return cleanup(rc);
+        B->etab.add(bases[m]);
+    }
+    if (int rc = B->etab.build(ctx->stream)) return cleanup(rc);
+    for (int m = 0; m < n_mol; m++) {
         hf_system* s = nullptr;
-        int rc = hf_system_create(ctx, &geoms[m], &bases[m], &t, &s);
+        int rc = create_system(ctx, &geoms[m], &bases[m], &t, &B->etab, &s);
         if (rc != HF_OK) return cleanup(rc);
         B->sys.push_back(s);
     }
@@ -273,10 +285,9 @@ int hf_batch_create(hf_ctx* ctx, int n_mol, const hf_geometry* geoms, const hf_b
             hf_system* s = B->sys[m];
             MolClass& d = mc[m];
             memset(&d, 0, sizeof(d));
-            d.pairs = s->pairs.as<PairHdr>();
-            d.prims64 = s->prims64.p;
-            d.bra = s->class_ids[Xc].as<int>();
-            d.ket = s->class_ids[Yc].as<int>();
+            d.bhdr = s->class_hdr[Xc].as<PairHdr>();
+            d.khdr = s->class_hdr[Yc].as<PairHdr>();
+            d.herm = s->herm;
             d.offsets = s->plan[c].offsets64.as<long long>();
             d.n_bra = s->class_count[Xc];
             d.same = Xc == Yc;
@@ -404,7 +415,7 @@ int hf_batch_tune(hf_batch* B, const char* cache_path, int64_t sample_quartets)
     for (int c = 0; c < kNumClasses; c++) {
         if (have[c] || B->n_total[c] <= 0) continue;
         // sample about 2e10 algorithmic operations per candidate launch (a few ms), at most sample_quartets
-        const double per_quartet = 81.0 * kEriClasses[c].prim_flops + kEriClasses[c].cont_flops;
+        const double per_quartet = 81.0 * kEriClasses[c].prim_flops_h + kEriClasses[c].cont_flops_h;
         long long limit = (long long)(2e10 / per_quartet);
         limit = std::max(2048LL, std::min(limit, sample_quartets > 0 ? (long long)sample_quartets : 2000000LL));
         float best = 1e30f;
@@ -415,10 +426,10 @@ int hf_batch_tune(hf_batch* B, const char* cache_path, int64_t sample_quartets)
                     BatchArgs a = batch_args(B, c, limit);
                     a.chunk = ch;
                     HF_CUDA(cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), st));
-                    kEriClasses[c].launch_batch(a, B->num_sms * bp, bl, st);  // warm-up
+                    kEriClasses[c].launch_batch(a, batch_grid(B, c, bp), bl, st);  // warm-up
                     HF_CUDA(cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), st));
                     HF_CUDA(cudaEventRecord(B->t0, st));
-                    kEriClasses[c].launch_batch(a, B->num_sms * bp, bl, st);
+                    kEriClasses[c].launch_batch(a, batch_grid(B, c, bp), bl, st);
                     HF_CUDA(cudaEventRecord(B->t1, st));
                     HF_CUDA(cudaEventSynchronize(B->t1));
                     HF_CUDA(cudaGetLastError());

@@ -53,6 +53,32 @@ void DevBuf::release()
     owned = true;
 }
 
+void ExponentTable::add(const hf_basis& b)
+{
+    long long n = 0;
+    for (int s = 0; s < b.n_shells; s++) n += b.nprim[s];
+    exps.insert(exps.end(), b.exps, b.exps + n);
+    std::sort(exps.begin(), exps.end());
+    exps.erase(std::unique(exps.begin(), exps.end()), exps.end());
+}
+
+int ExponentTable::build(cudaStream_t s)
+{
+    const long long n = (long long)exps.size(), nt = n * (n + 1) / 2;
+    if (nt > kHermMaxTypes) return HF_OK;
+    std::vector<double> ps;
+    for (int i = 0; i < n; i++)
+        for (int j = 0; j <= i; j++) ps.push_back(exps[i] + exps[j]);  // type i (i + 1) / 2 + j
+    int rc = psum.alloc(sizeof(double) * nt);
+    if (rc == HF_OK) rc = tab.alloc(sizeof(double2) * nt * nt);
+    if (rc != HF_OK) return rc;
+    HF_CUDA(cudaMemcpyAsync(psum.p, ps.data(), sizeof(double) * nt, cudaMemcpyHostToDevice, s));
+    HF_CUDA(cudaStreamSynchronize(s));  // ps goes out of scope
+    ntype = (int)nt;
+    return launch_exponent_table(ntype, psum.as<double>(), tab.as<double2>(), s) == 0
+               ? HF_OK : cuda_status(cudaGetLastError(), "exponent table");
+}
+
 namespace {
 
 struct DeviceGuard {
@@ -171,6 +197,8 @@ int hf_create(hf_ctx** out, int device, void* cuda_stream)
         for (int ci = 0; ci < kNumClasses; ci++) {
             need = std::max(need, kEriClasses[ci].local_bytes());
             if (kEriClasses[ci].local_bytes_rys) need = std::max(need, kEriClasses[ci].local_bytes_rys());
+            need = std::max(need, kEriClasses[ci].local_bytes_h());
+            if (kEriClasses[ci].prepare() != 0) rc = cuda_status(cudaGetLastError(), "hf_create: shared memory limit");
         }
         size_t cur = 0;
         if (cudaDeviceGetLimit(&cur, cudaLimitStackSize) == cudaSuccess && need > cur)
@@ -236,7 +264,7 @@ struct Arena {
     }
 };
 
-static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* basis)
+static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* basis, const ExponentTable* shared)
 {
     hf_ctx* ctx = S->ctx;
     cudaStream_t st = ctx->stream;
@@ -283,7 +311,18 @@ static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* b
     S->n_pairs_all = (int)npairs;
     const size_t NN = (size_t)nbf * nbf;
 
+    // exponent table and each primitive's place in it
+    if (!shared) {
+        S->etab.add(*basis);
+        TRY(S->etab.build(st));
+        shared = &S->etab;
+    }
+    std::vector<int> utype(npr);
+    for (int k = 0; k < npr; k++)
+        utype[k] = (int)(std::lower_bound(shared->exps.begin(), shared->exps.end(), basis->exps[k]) - shared->exps.begin());
+
     // ---------------------------------------------- inputs, matrices, pairs
+    DevBuf utype_in;
     DevBuf coef_in;
     Arena a1;
     a1.add(S->sh_l, sizeof(int) * ns);
@@ -301,6 +340,9 @@ static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* b
     a1.add(S->pairs, sizeof(PairHdr) * npairs);
     a1.add(S->prims64, sizeof(PrimPair<double>) * npairs * X.maxpp);
     a1.add(S->prims32, sizeof(PrimPair<float>) * npairs * X.maxpp);
+    a1.add(utype_in, sizeof(int) * npr);
+    a1.add(S->hrec, sizeof(HermPair) * npairs * X.maxpp);
+    a1.add(S->hB, sizeof(float) * npairs * X.maxpp);
     a1.add(S->pair_class, sizeof(int) * npairs);
     a1.add(X.counts, sizeof(unsigned long long) * 16);
     a1.add(X.Qall, sizeof(double) * npairs);
@@ -328,6 +370,11 @@ static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* b
     HF_CUDA(cudaMemcpyAsync(coef_in.p, basis->coefs, sizeof(double) * npr, cudaMemcpyHostToDevice, st));
     HF_CUDA(cudaMemcpyAsync(S->atom_xyz.p, geom->xyz, sizeof(double) * 3 * na, cudaMemcpyHostToDevice, st));
     HF_CUDA(cudaMemcpyAsync(S->atom_Z.p, Zd.data(), sizeof(double) * na, cudaMemcpyHostToDevice, st));
+    HF_CUDA(cudaMemcpyAsync(utype_in.p, utype.data(), sizeof(int) * npr, cudaMemcpyHostToDevice, st));
+    HF_CUDA(cudaMemsetAsync(S->hB.p, 0, sizeof(float) * npairs * X.maxpp, st));
+    S->herm.rec = S->hrec.as<HermPair>();
+    S->herm.B = S->hB.as<float>();
+    S->herm = shared->view(S->herm);
     KCHK(launch_shell_coef(ns, S->sh_l.as<int>(), S->sh_nprim.as<int>(), S->sh_prim0.as<int>(), S->sh_exp.as<double>(),
                            coef_in.as<double>(), S->sh_coef.as<double>(), st));
     KCHK(launch_comp_norm(ns, S->sh_l.as<int>(), S->sh_bf0.as<int>(), S->comp_norm.as<double>(), st));
@@ -341,7 +388,8 @@ static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* b
     KCHK(launch_build_pairs(npairs, X.maxpp, S->sh_l.as<int>(), S->sh_atom.as<int>(), S->sh_bf0.as<int>(),
                             S->sh_nprim.as<int>(), S->sh_prim0.as<int>(), S->sh_exp.as<double>(),
                             S->sh_coef.as<double>(), S->atom_xyz.as<double>(), S->pairs.as<PairHdr>(),
-                            S->prims64.p, S->prims32.p, S->pair_class.as<int>(), st));
+                            S->prims64.p, S->prims32.p, S->hrec.as<HermPair>(), utype_in.as<int>(),
+                            S->pair_class.as<int>(), st));
     unsigned long long* cnt_dev = X.counts.as<unsigned long long>();  // [0..5] class counts, [8..15] cursors
     HF_CUDA(cudaMemsetAsync(cnt_dev, 0, sizeof(unsigned long long) * 16, st));
     KCHK(launch_class_count(npairs, S->pair_class.as<int>(), cnt_dev, st));
@@ -388,7 +436,7 @@ static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* b
         KCHK(launch_class_scatter_all(npairs, S->pair_class.as<int>(), c, (unsigned*)(cnt_dev + 8 + c), ids, st));
         SchwarzArgs sa;
         sa.pairs = S->pairs.as<PairHdr>();
-        sa.prims64 = S->prims64.p;
+        sa.herm = S->herm;
         sa.ids = ids;
         sa.n = (int)cnt_all[c];
         sa.Q = X.Qall.as<double>();
@@ -398,7 +446,8 @@ static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* b
         kEriClasses[class_index(c, c)].launch_schwarz(sa, kEriThreads, st);
         HF_CUDA(cudaGetLastError());
     }
-    KCHK(launch_sort_prims(npairs, S->pairs.as<PairHdr>(), X.Bprim.as<double>(), S->prims64.p, S->prims32.p, st));
+    KCHK(launch_sort_prims(npairs, S->pairs.as<PairHdr>(), X.Bprim.as<double>(), S->prims64.p, S->prims32.p,
+                           S->hrec.as<HermPair>(), S->hB.as<float>(), st));
     unsigned long long* qbits_dev = cnt_dev + 7;
     HF_CUDA(cudaMemsetAsync(qbits_dev, 0, sizeof(unsigned long long), st));
     KCHK(launch_copy_q(npairs, X.Qall.as<double>(), S->pairs.as<PairHdr>(), qbits_dev, st));
@@ -482,7 +531,7 @@ static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* b
     return HF_OK;
 }
 
-static int check_geometry_basis(const hf_geometry* g, const hf_basis* b, const hf_thresholds* th)
+int hf::check_geometry_basis(const hf_geometry* g, const hf_basis* b, const hf_thresholds* th)
 {
     if (!g || !b) return fail(HF_E_INVALID, "geometry or basis is NULL");
     if (g->n_atoms < 1 || !g->Z || !g->xyz) return fail(HF_E_INVALID, "geometry: empty or NULL arrays");
@@ -564,13 +613,9 @@ static const hf_basis* expand_sp_shells(const hf_basis* b, ExpandedBasis& e)
     return &e.view;
 }
 
-extern "C" {
-
-int hf_system_create(hf_ctx* ctx, const hf_geometry* geom, const hf_basis* basis_in, const hf_thresholds* th,
-                     hf_system** out)
+int hf::create_system(hf_ctx* ctx, const hf_geometry* geom, const hf_basis* basis_in, const hf_thresholds* th,
+                      const ExponentTable* shared, hf_system** out)
 {
-    if (!ctx || !out) return fail(HF_E_INVALID, "hf_system_create: NULL ctx or output pointer");
-    *out = nullptr;
     TRY(check_geometry_basis(geom, basis_in, th));
     ExpandedBasis eb;
     const hf_basis* basis = expand_sp_shells(basis_in, eb);
@@ -580,7 +625,7 @@ int hf_system_create(hf_ctx* ctx, const hf_geometry* geom, const hf_basis* basis
     S->device = ctx->device;
     S->stream = ctx->stream;
     if (th) S->th = *th;
-    int rc = system_setup(S, geom, basis);
+    int rc = system_setup(S, geom, basis, shared);
     if (rc != HF_OK) {
         cudaStreamSynchronize(ctx->stream);
         delete S;
@@ -589,6 +634,16 @@ int hf_system_create(hf_ctx* ctx, const hf_geometry* geom, const hf_basis* basis
     ctx->n_systems++;
     *out = S;
     return HF_OK;
+}
+
+extern "C" {
+
+int hf_system_create(hf_ctx* ctx, const hf_geometry* geom, const hf_basis* basis, const hf_thresholds* th,
+                     hf_system** out)
+{
+    if (!ctx || !out) return fail(HF_E_INVALID, "hf_system_create: NULL ctx or output pointer");
+    *out = nullptr;
+    return create_system(ctx, geom, basis, th, nullptr, out);
 }
 
 void hf_system_destroy(hf_system* S)
@@ -624,7 +679,7 @@ int hf_system_get_info(const hf_system* S, hf_system_info* info)
     const DevBuf* bufs[] = {&S->sh_l, &S->sh_atom, &S->sh_bf0, &S->sh_nprim, &S->sh_prim0, &S->sh_exp, &S->sh_coef,
                             &S->atom_xyz, &S->atom_Z, &S->comp_norm, &S->pairs, &S->prims64, &S->prims32,
                             &S->pair_class, &S->S, &S->H, &S->P64, &S->P32, &S->Jt, &S->Kt, &S->F, &S->Ebuf,
-                            &S->Qall, &S->staging_P, &S->staging_out};
+                            &S->Qall, &S->staging_P, &S->staging_out, &S->hrec, &S->hB, &S->etab.tab};
     for (auto* b : bufs) bytes += b->bytes;
     for (int c = 0; c < kNumPairClasses; c++)
         bytes += S->class_ids[c].bytes + S->class_q[c].bytes + S->ket_tab[c].bytes + S->class_hdr[c].bytes;
@@ -705,17 +760,13 @@ int hf_system_set_fock_copies(hf_system* S, int32_t copies)
 
 }  // extern "C"
 
-// Whether a launch of class ci runs the Rys-quadrature kernel: an FP64 launch of a class whose Rys variant
-// the flags select (class_uses_rys), with the ket tables in use.
-static bool uses_rys(int ci, int flags, int use_f32, const EriArgs& a)
-{
-    return !use_f32 && class_uses_rys(ci, flags) && a.kt;
-}
-// (the ket tables always exist for a class with significant pairs, so a.kt is set for every launch)
-
 // One class launch of a build.
 struct ClassLaunch {
-    int ci, prec, use_f32, lanes, grid;
+    int ci, prec, use_f32;
+    Fp64Method method;
+    bool warp;   // Hermite warp kernel
+    int lanes;   // lanes per quartet (thread kernels), parts per quartet (warp kernel)
+    int grid;
     double est;  // estimated device time, in operations of the whole GPU
 };
 
@@ -739,21 +790,38 @@ int hf::launch_eri_classes(hf_system* S, EriArgs a, int shard, int n_shards, int
     a.boys64 = ctx->boys64.as<double>();
     a.boys32 = ctx->boys32.as<float>();
     a.prim_tau = S->th.prim_tau;
+    a.herm = S->herm;
     ClassLaunch todo[2 * kNumClasses];
     int n_todo = 0;
     for (int ci = 0; ci < kNumClasses; ci++)
         for (int prec = 0; prec < 2; prec++) {
             const long long n = prec ? S->plan[ci].n32 : S->plan[ci].n64;
             const long long nq = n * (shard + 1) / n_shards - n * shard / n_shards;
-            ClassLaunch c{ci, prec, prec && !(flags & HF_FP64_ONLY), 1, 0, 0.0};
+            const EriClassEntry& cl = kEriClasses[ci];
+            ClassLaunch c{ci, prec, prec && !(flags & HF_FP64_ONLY), fp64_method(ci, flags), false, 1, 0, 0.0};
+            const bool herm = !c.use_f32 && c.method == Fp64Method::kHerm;
             // a class too small to fill the GPU with one thread per quartet shares each quartet's
-            // primitive work among a lane group instead (shorter latency, same result)
-            if (!c.use_f32 && nq < (long long)ctx->num_sms * 256) c.lanes = kEriClasses[ci].lanes;
-            const long long blocks = (nq * c.lanes + kEriThreads - 1) / kEriThreads;
-            c.grid = (int)std::min<long long>(blocks, (long long)ctx->num_sms * 16);
-            // one quartet's operations run in one lane group, 1 / (64 lanes SMs) of the GPU at a time
-            const double ops = (double)kEriClasses[ci].prim_flops * X.maxpp * X.maxpp / c.lanes + kEriClasses[ci].cont_flops;
-            c.est = std::max((double)nq * c.lanes, 64.0 * ctx->num_sms) * ops / (c.use_f32 ? 32.0 : 1.0);
+            // primitive work among a lane group or a warp instead (shorter latency, same result)
+            const bool small = !c.use_f32 && nq < (long long)ctx->num_sms * 256;
+            double ops = (double)cl.prim_flops * X.maxpp * X.maxpp + cl.cont_flops;
+            if (herm) {
+                ops = (double)cl.prim_flops_h * X.maxpp * X.maxpp + cl.cont_flops_h;
+                c.warp = !cl.launch_herm || (small && cl.launch_hermw);
+                if (c.warp) {
+                    // parts: quartets fewer than four warps per SM take one warp per batch of 32 primitive quartets
+                    const long long batches = ((long long)X.maxpp * X.maxpp + 31) / 32;
+                    c.lanes = (int)std::max<long long>(1, std::min(batches, (long long)ctx->num_sms * 4 / std::max<long long>(nq, 1)));
+                    c.grid = (int)std::min<long long>(nq * c.lanes, 1 << 20);
+                } else if (small) {
+                    c.lanes = cl.herm_lanes;
+                }
+            } else if (small) {
+                c.lanes = cl.lanes;
+            }
+            if (!c.warp)
+                c.grid = (int)std::min<long long>((nq * c.lanes + kEriThreads - 1) / kEriThreads, (long long)ctx->num_sms * 16);
+            // one quartet's operations run in one lane (warp), 1 / (64 lanes SMs) of the GPU at a time
+            c.est = std::max((double)nq, 64.0 * ctx->num_sms / (c.warp ? 32 * c.lanes : c.lanes)) * ops / (c.use_f32 ? 32.0 : 1.0);
             if (nq > 0 || ev) todo[n_todo++] = c;
         }
     const bool forked = !ev && n_todo > 1;
@@ -804,10 +872,15 @@ int hf::launch_eri_classes(hf_system* S, EriArgs a, int shard, int n_shards, int
             // 2% faster); the FP32 kernels, bound by latency rather than a pipe, ran 10% slower with it
             // and are compiled without it
             a.sort_work = c.use_f32 ? 0 : 1;
-            if (uses_rys(c.ci, flags, c.use_f32, a))
-                kEriClasses[c.ci].launch_rys(a, 0, c.grid, kEriThreads, st, c.lanes);
+            const EriClassEntry& cl = kEriClasses[c.ci];
+            if (c.use_f32 || c.method == Fp64Method::kObaraSaika)
+                cl.launch(a, c.use_f32, c.grid, kEriThreads, st, c.lanes);
+            else if (c.method == Fp64Method::kRys)
+                cl.launch_rys(a, 0, c.grid, kEriThreads, st, c.lanes);
+            else if (c.warp)
+                cl.launch_hermw(a, c.grid, st, c.lanes);
             else
-                kEriClasses[c.ci].launch(a, c.use_f32, c.grid, kEriThreads, st, c.lanes);
+                cl.launch_herm(a, c.grid, st, c.lanes);
             err = cudaGetLastError();
         }
         if (ev && err == cudaSuccess) err = cudaEventRecord(ev[4 * c.ci + 2 * c.prec + 1], st);
@@ -894,12 +967,15 @@ int hf_fock_build(hf_system* S, const double* P, double* F, double* J, double* K
             stats->quartets_fp32 += pl.n32;
             stats->prim_quartets_fp64 += (int64_t)pc[2 * ci];
             stats->prim_quartets_fp32 += (int64_t)pc[2 * ci + 1];
-            const double pf = kEriClasses[ci].prim_flops, cf = kEriClasses[ci].cont_flops;
-            const bool rys = class_uses_rys(ci, flags);
-            const double pf64 = rys ? kEriClasses[ci].prim_flops_rys : pf;
-            const double pf32 = (rys && (flags & HF_FP64_ONLY)) ? pf64 : pf;  // FP32 launches stay Obara-Saika
-            stats->class_flops_fp64[ci] = pf64 * (double)pc[2 * ci] + cf * (double)pl.n64;
-            stats->class_flops_fp32[ci] = pf32 * (double)pc[2 * ci + 1] + cf * (double)pl.n32;
+            const EriClassEntry& cl = kEriClasses[ci];
+            const Fp64Method m = fp64_method(ci, flags);
+            const bool herm = m == Fp64Method::kHerm;
+            const double pf64 = herm ? cl.prim_flops_h : m == Fp64Method::kRys ? cl.prim_flops_rys : cl.prim_flops;
+            const double cf64 = herm ? cl.cont_flops_h : cl.cont_flops;
+            const bool f64 = (flags & HF_FP64_ONLY) != 0;  // else FP32 launches, which are Obara-Saika
+            stats->class_flops_fp64[ci] = pf64 * (double)pc[2 * ci] + cf64 * (double)pl.n64;
+            stats->class_flops_fp32[ci] = (f64 ? pf64 : cl.prim_flops) * (double)pc[2 * ci + 1] +
+                                          (f64 ? cf64 : cl.cont_flops) * (double)pl.n32;
             stats->flops_fp64 += stats->class_flops_fp64[ci];
             stats->flops_fp32 += stats->class_flops_fp32[ci];
             stats->kernels_launched += (pl.n64 > 0) + (pl.n32 > 0);

@@ -80,8 +80,8 @@ constexpr int kBoysBinade0 = 6;    // region B starts at 2^6 = 64
 constexpr int kBoysBinades = 26;   // binades 2^6 .. 2^31 (the last one only its first row)
 constexpr int kBoysSubBits = 12;   // 4096 rows per binade
 constexpr int kBoysRows64 = kBoysRowsA + (kBoysBinades << kBoysSubBits);
-constexpr long long kBoysBitsB = 0x4050000000000000LL;    // bit pattern of 64.0
-constexpr long long kBoysBitsTop = 0x41E0000000000000LL;  // bit pattern of 2^31
+constexpr int kBoysHiB = 0x40500000;    // high word of 64.0
+constexpr int kBoysHiTop = 0x41E00000;  // high word of 2^31
 constexpr int kBoysRows32 = 60 * 32 + 1;
 constexpr int kBoysStride64 = 50;
 constexpr int kBoysStride32 = 44;
@@ -108,33 +108,44 @@ __host__ __device__ constexpr float boys_switch32(int L)
          : L == 6 ? 31.0f : L == 7 ? 33.0f : 35.0f;
 }
 
+// Table row of T < 2^31 and its grid point T_k, from the high word of T in integer arithmetic: both regions
+// round T to its leading mantissa bits (region A: to a multiple of 1/512; region B: to 12 bits), so dropping s
+// bits of the high word after adding half a unit gives T_k's high word (a carry moves into the exponent, as it
+// should) and the row index.  The ERI kernels are bound by FP64 instructions; this leaves one of them
+// (d = T_k - T) where the 1.5 * 2^52 trick and the region select took four.
+__device__ __forceinline__ int boys_row(double T, double& Tk)
+{
+    const int h = __double2hiint(T);
+    const bool regb = h >= kBoysHiB;
+    const int s = regb ? 20 - kBoysSubBits : min(11 + 1023 - (h >> 20), 20);
+    const int half = 1 << (s - 1);
+    int hr = (h + half) & (int)(0xffffffffu << s);
+    int k = ((h & 0xfffff) + 0x100000 + half) >> s;
+    if (h < 0x3F600000) {  // T < 1/512: row 0 or 1
+        k = h >= 0x3F500000;
+        hr = k ? 0x3F600000 : 0;
+    }
+    if (regb) k = (hr >> (20 - kBoysSubBits)) - (kBoysHiB >> (20 - kBoysSubBits)) + kBoysRowsA;
+    Tk = __hiloint2double(hr, 0);
+    return k;
+}
+
 // F_m(T), m = 0..L, FP64.  Taylor expansion about the nearest row T_k of the table (region A: |T - T_k| <=
 // 1/1024, five terms, truncation below (1/1024)^5 / 5! < 1e-17 relative, as |F_{m+5}| <= |F_m|; region B:
 // |T - T_k| <= T / 8192, where the asymptotic form's fifth-order term is below 2e-17 relative for m <= 8),
 // using dF_m/dT = -F_{m+1}, which the asymptotic form obeys as well.  For L >= 2 only F_L is expanded and
 // the rest follow from the downward recursion F_m = (2T F_{m+1} + e^{-T}) / (2m+1), with e^{-T} =
-// e^{-T_k} e^{T_k - T} expanded the same way (zero in region B).  Region A's row is the integer that
-// T*512 + 1.5*2^52 rounds to, read from the low word of the sum; region B's row and T_k come from T's bit
-// pattern rounded to 12 mantissa bits.  T >= 2^31 (far beyond any screened quartet) takes the asymptotic
+// e^{-T_k} e^{T_k - T} expanded the same way (zero in region B).  boys_row gives the row and T_k from T's
+// bits.  T >= 2^31 (far beyond any screened quartet) takes the asymptotic
 // form directly: F_0 = sqrt(pi/T)/2, F_{m+1} = (2m+1) F_m / (2T).
 static_assert(boys_switch64(8) <= 64.0, "region B of the FP64 table must lie above every switch point");
 template <int L>
 __device__ __forceinline__ void boys_eval(double T, const double* __restrict__ tab, double* F)
 {
-    const long long bits = __double_as_longlong(T);
-    if (bits < kBoysBitsTop) {
-        const double big = 6755399441055744.0;  // 1.5 * 2^52
-        const double t = fma(T, 512.0, big);
-        int k = __double2loint(t);
-        double d = fma(t - big, 1.0 / 512.0, -T);  // T_k - T (region A)
-        const long long rb = bits + (1LL << (51 - kBoysSubBits));
-        const double Tk = __longlong_as_double(rb & ~((1LL << (52 - kBoysSubBits)) - 1));
-        const double dB = Tk - T;
-        if (bits >= kBoysBitsB) {
-            k = kBoysRowsA + (((int)(rb >> 52) - 1023 - kBoysBinade0) << kBoysSubBits)
-              + (int)((rb >> (52 - kBoysSubBits)) & ((1 << kBoysSubBits) - 1));
-            d = dB;
-        }
+    if (__double2hiint(T) < kBoysHiTop) {
+        double Tk;
+        const int k = boys_row(T, Tk);
+        const double d = Tk - T;
         const double* __restrict__ r = tab + (size_t)k * kBoysStride64;
         if constexpr (L <= 1) {
 #pragma unroll
@@ -422,7 +433,7 @@ __device__ __forceinline__ void warp_bitonic_sort(unsigned* k, int n, int lane32
         cudaFuncAttributes fa;                                                                               \
         size_t m = 0;                                                                                        \
         const void* fns[] = {(const void*)k_eri_##NAME<double, 1, false>, (const void*)k_eri_##NAME<double, (GL), false>, \
-                             (const void*)k_eri_##NAME<float, 1, true>, (const void*)k_eri_batch_##NAME};   \
+                             (const void*)k_eri_##NAME<float, 1, true>};                                     \
         for (const void* fn : fns)                                                                           \
             if (cudaFuncGetAttributes(&fa, fn) == cudaSuccess && fa.localSizeBytes > m) m = fa.localSizeBytes; \
         cudaGetLastError();                                                                                  \
@@ -451,85 +462,4 @@ __device__ __forceinline__ void warp_bitonic_sort(unsigned* k, int n, int lane32
             m = fa.localSizeBytes;                                                                           \
         cudaGetLastError();                                                                                  \
         return m;                                                                                            \
-    }
-
-// Schwarz bounds of the pairs of a diagonal class: Q = sqrt(max |(ab|ab)|) of the
-// contracted pair (item 0 of each pair) and B = the same bound of each primitive pair
-// alone (items 1..a.items-1), one thread per item so that the high-L classes'
-// single-thread latency is paid once per pair, not once per primitive pair.
-#define SCHWARZ_KERNEL(NAME)                                                                                 \
-    __global__ void __launch_bounds__(kEriThreads) k_schwarz_##NAME(const SchwarzArgs a)                    \
-    {                                                                                                        \
-        const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;                                \
-        if (t >= (long long)a.n * a.items) return;                                                           \
-        const int pid = a.ids[t / a.items];                                                                  \
-        const int item = (int)(t % a.items);                                                                 \
-        PairHdr h = a.pairs[pid];                                                                            \
-        if (item > h.nprim) return;                                                                          \
-        const PrimPair<double>* pr = (const PrimPair<double>*)a.prims64;                                     \
-        if (item > 0) { /* bound of one primitive pair alone */                                              \
-            h.prim0 += item - 1;                                                                             \
-            h.nprim = 1;                                                                                     \
-        }                                                                                                    \
-        double qm = 0.0;                                                                                     \
-        quartet_##NAME<double, 1>(h, h, KetAos<double>{pr + h.prim0}, pr, a.boys64, nullptr, 0, 1.0, nullptr,  \
-                                  nullptr, &qm, 0.0f, 0, true);                                              \
-        if (item == 0)                                                                                       \
-            a.Q[pid] = sqrt(qm);                                                                             \
-        else                                                                                                 \
-            a.Bprim[h.prim0] = sqrt(qm);                                                                     \
-    }                                                                                                        \
-    void launch_schwarz_##NAME(const SchwarzArgs& a, int block, cudaStream_t s)                             \
-    {                                                                                                        \
-        const long long items = (long long)a.n * a.items;                                                    \
-        if (items > 0) k_schwarz_##NAME<<<(unsigned)((items + block - 1) / block), block, 0, s>>>(a);        \
-    }
-
-// Batched build: one persistent kernel per class over many molecules.  Warps
-// take chunks of the batch's quartet index space from a device counter (the
-// GPU analogue of the paper's dynamic load balancing, ddi_dlbnext); a quartet
-// index resolves to (molecule, bra, ket) by two binary searches.
-#define ERI_BATCH_KERNEL(NAME, GL_UNUSED)                                                                           \
-    __global__ void __launch_bounds__(256) k_eri_batch_##NAME(const BatchArgs a)                            \
-    {                                                                                                        \
-        const int wl = threadIdx.x & 31;                                                                     \
-        constexpr int GL = 1; /* batches have enough quartets per class for one thread per quartet */        \
-        const int lane = 0;                                                                                  \
-        const int grp = wl;                                                                                  \
-        constexpr int gpw = 32;                                                                              \
-        const float ptau = (float)a.prim_tau;                                                                \
-        for (;;) {                                                                                           \
-            unsigned long long base = 0;                                                                     \
-            if (wl == 0) base = atomicAdd(a.counter, (unsigned long long)a.chunk);                          \
-            base = __shfl_sync(0xffffffffu, base, 0);                                                        \
-            if (base >= (unsigned long long)a.n_total) break;                                                \
-            const long long end = min((long long)base + a.chunk, a.n_total);                                 \
-            for (long long wq = (long long)base; wq < end; wq += gpw) { /* warp-uniform */                  \
-                const long long q = wq + grp;                                                                \
-                const bool valid = q < end;                                                                  \
-                const int m = find_bra(a.mol_off, a.n_mol, valid ? q : (long long)base);                     \
-                const MolClass mc = a.mols[m];                                                               \
-                PairHdr hb, hk;                                                                              \
-                double f = 1.0;                                                                              \
-                if (valid) {                                                                                 \
-                    const long long ql = q - a.mol_off[m];                                                   \
-                    const int b = find_bra(mc.offsets, mc.n_bra, ql);                                        \
-                    const int k = (int)(ql - mc.offsets[b]);                                                 \
-                    hb = mc.pairs[mc.bra[b]];                                                                \
-                    hk = mc.pairs[mc.ket[k]];                                                                \
-                    if (hb.A == hb.B) f *= 0.5;                                                              \
-                    if (hk.A == hk.B) f *= 0.5;                                                              \
-                    if (mc.same && b == k) f *= 0.5;                                                         \
-                } else {                                                                                     \
-                    hb = hk = mc.pairs[mc.bra[0]];                                                           \
-                }                                                                                            \
-                const PrimPair<double>* mp = (const PrimPair<double>*)mc.prims64;                            \
-                quartet_##NAME<double, (GL)>(hb, hk, KetAos<double>{mp + hk.prim0}, mp, a.boys64, mc.P64, mc.N, f, \
-                                             mc.Jt, mc.Kt, nullptr, ptau, lane, valid);                      \
-            }                                                                                                \
-        }                                                                                                    \
-    }                                                                                                        \
-    void launch_eri_batch_##NAME(const BatchArgs& a, int grid, int block, cudaStream_t s)                   \
-    {                                                                                                        \
-        k_eri_batch_##NAME<<<grid, block, 0, s>>>(a);                                                        \
     }

@@ -36,7 +36,8 @@ from __future__ import annotations
 
 import json
 import os
-import sys
+
+import gen_herm
 
 CART = {L: [(x, y, L - x - y) for x in range(L, -1, -1) for y in range(L - x, -1, -1)] for L in range(9)}
 PAIR_CLASSES = [(0, 0), (1, 0), (1, 1), (2, 0), (2, 1), (2, 2)]
@@ -235,9 +236,6 @@ def gen_vrr(la, lb, lc, ld, cnt, subset=None):
 
 
 RYS_MIN_L = 6  # classes that have a Rys-quadrature variant (all of them with HF_RYS)
-# Classes whose FP64 launches use the Rys variant by default (neither HF_RYS nor HF_OBARA_SAIKA given): those
-# where it measured faster than the Obara-Saika kernel on the 64-water build ((dd|pp) measured slower).
-RYS_DEFAULT = {"2121", "2220", "2221", "2222"}
 FOLD = True  # fold rho/p (rho/q) into the recurrence values when that saves multiplies
 
 
@@ -734,12 +732,66 @@ def gen_class(X, Y, method="os"):
     if method == "rys":
         out.append(f"ERI_RYS_KERNELS({name}, {G})")
     else:
-        out.append(f"ERI_BATCH_KERNEL({name}, {G})")
         out.append(f"ERI_CLASS_KERNELS({name}, {X}, {Y}, {G})")
-        if X == Y:
-            out.append(f"SCHWARZ_KERNEL({name})")
     info = dict(name=name, X=X, Y=Y, l=[la, lb, lc, ld], L=L, G=G, prim_flops=prim_flops, cont_flops=cnt.cont,
                 hrr_flops=cont_hrr, targets=len(targets), vrr_nodes=len(vrr))
+    return "\n".join(out) + "\n", info
+
+
+# Hermite-accumulator kernels: classes up to this total angular momentum have a thread kernel (their
+# accumulators fit the registers, with a few spills at 100 to 157 of them), classes from HERM_WARP_MIN_L on a
+# warp kernel; small launches of the classes with both use the warp kernel.
+HERM_THREAD_MAX_L = 4
+HERM_WARP_MIN_L = 4
+HERM_LANES = 8  # lanes per quartet of the thread kernels in small launches and Schwarz bounds
+
+
+def gen_herm_class(X, Y):
+    """Source of one class's Hermite-accumulator kernels."""
+    la, lb = PAIR_CLASSES[X]
+    lc, ld = PAIR_CLASSES[Y]
+    L = la + lb + lc + ld
+    name = class_name(X, Y)
+
+    def hrr_digest(final):
+        cnt = Counter()
+        lines = [f"const double acc{tstr(e)}_{tstr(f)} = {nm};" for (e, f), nm in final.items()]
+        hl, xname = gen_hrr(la, lb, lc, ld, cnt)
+        lines += hl
+        if X == Y:
+            lines.append("if (qout) {")
+            lines += ["    " + l for l in gen_schwarz(la, lb, xname)]
+            lines += ["    *qout = qmax;", "    return nq;", "}"]
+        lines.append("if (total == 0) return nq;  // every primitive quartet screened: nothing to digest")
+        lines.append("const int bA = hb.bfA, bB_ = hb.bfB, bC = hk.bfA, bD = hk.bfB;")
+        lines.append("const double fj = 4.0 * fscale, fk = 2.0 * fscale;")
+        dig = gen_digest(la, lb, lc, ld, xname, cnt)
+        lines += [l.replace("(bB +", "(bB_ +").replace("* N + bB +", "* N + bB_ +") for l in dig]
+        return lines, cnt.cont, None
+
+    out = [f"// ({PAIR_NAMES[X]}|{PAIR_NAMES[Y]}) class: l = {la}{lb}{lc}{ld}, Hermite accumulators."]
+    info = dict(hname=name, herm_thread=L <= HERM_THREAD_MAX_L, herm_warp=L >= HERM_WARP_MIN_L)
+    kernels = []
+    if info["herm_thread"]:
+        src, pf, cf, nacc = gen_herm.gen_thread(name, la, lb, lc, ld, hrr_digest)
+        out += [src, f"HERM_THREAD_KERNELS({name}, {HERM_LANES})", f"HERM_THREAD_BATCH({name})"]
+        kernels += [f"k_herm_{name}<1>", f"k_herm_{name}<{HERM_LANES}>"]
+        info.update(prim_flops_h=pf, cont_flops_h=cf)
+    if info["herm_warp"]:
+        src, pf, cf = gen_herm.gen_warp(name, la, lb, lc, ld)
+        out += [src, f"HERM_WARP_KERNELS({name})"]
+        kernels += [f"k_hermw_{name}"]
+        if not info["herm_thread"]:
+            out.append(f"HERM_WARP_BATCH({name})")
+            info.update(prim_flops_h=pf, cont_flops_h=cf)
+    kernels.append(f"k_eri_batch_{name}")
+    if X == Y:
+        out.append(f"{'HERM_WARP_SCHWARZ' if info['herm_warp'] else 'HERM_THREAD_SCHWARZ'}({name})")
+        kernels.append(f"k_schwarz_{name}")
+    prep = ([f"prepare_hermw_{name}()"] if info["herm_warp"] else []) + \
+           ([f"prepare_batch_{name}()"] if not info["herm_thread"] else [])
+    out.append(f"int prepare_herm_{name}() {{ return {' | '.join(prep) if prep else '0'}; }}")
+    out.append(f"size_t local_bytes_h_{name}() {{ return herm_local_bytes({', '.join(kernels)}); }}")
     return "\n".join(out) + "\n", info
 
 
@@ -772,11 +824,24 @@ def main(outdir):
             if not os.path.exists(path) or open(path).read() != text:
                 with open(path, "w") as fh:
                     fh.write(text)
+        hsrc, hinfo = gen_herm_class(X, Y)
+        info.update(hinfo)
+        path = os.path.join(outdir, f"eri_h_{info['name']}.cu")
+        text = HEADER.replace("eri_common.cuh", "eri_herm.cuh") + hsrc + FOOTER
+        if not os.path.exists(path) or open(path).read() != text:
+            with open(path, "w") as fh:
+                fh.write(text)
     # dispatch table
     lines = ['// Generated by gen_eri.py: do not edit.', '#include "eri_common.cuh"', "", "namespace hf {"]
     for info in infos:
         n = info["name"]
         lines.append(f"void launch_eri_{n}(const EriArgs&, int, int, int, cudaStream_t, int);")
+        lines.append(f"int prepare_herm_{n}();")
+        lines.append(f"size_t local_bytes_h_{n}();")
+        if info["herm_thread"]:
+            lines.append(f"void launch_herm_{n}(const EriArgs&, int, cudaStream_t, int);")
+        if info["herm_warp"]:
+            lines.append(f"void launch_hermw_{n}(const EriArgs&, int, cudaStream_t, int);")
         if info["X"] == info["Y"]:
             lines.append(f"void launch_schwarz_{n}(const SchwarzArgs&, int, cudaStream_t);")
         lines.append(f"void launch_eri_batch_{n}(const BatchArgs&, int, int, cudaStream_t);")
@@ -788,12 +853,15 @@ def main(outdir):
     lines.append("const EriClassEntry kEriClasses[kNumClasses] = {")
     for info in infos:
         n = info["name"]
-        lines.append(f"    {{{info['X']}, {info['Y']}, {info['L']}, {info['prim_flops']}, {info['cont_flops']}, "
+        herm = (f"{info['prim_flops_h']}, {info['cont_flops_h']}, "
+                + (f"launch_herm_{n}" if info["herm_thread"] else "nullptr") + f", {HERM_LANES}, "
+                + (f"launch_hermw_{n}" if info["herm_warp"] else "nullptr")
+                + f", prepare_herm_{n}, local_bytes_h_{n}, {0 if info['herm_thread'] else 1}")
+        lines.append(f"    {{{info['X']}, {info['Y']}, {info['L']}, {herm}, {info['prim_flops']}, {info['cont_flops']}, "
                      f"launch_eri_{n}, {('launch_schwarz_' + n) if info['X'] == info['Y'] else 'nullptr'}, \"{n}\", "
                      f"launch_eri_batch_{n}, local_bytes_{n}, {info['G']}, "
-                     + (f"launch_eri_rys_{n}, {info['prim_flops_rys']}, local_bytes_rys_{n}, "
-                        f"{1 if n in RYS_DEFAULT else 0}}}," if info["rys"]
-                        else "nullptr, 0, nullptr, 0},"))
+                     + (f"launch_eri_rys_{n}, {info['prim_flops_rys']}, local_bytes_rys_{n}}}," if info["rys"]
+                        else "nullptr, 0, nullptr},"))
     lines.append("};")
     lines.append("}  // namespace hf")
     text = "\n".join(lines) + "\n"

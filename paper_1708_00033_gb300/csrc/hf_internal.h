@@ -28,6 +28,26 @@ struct PairHdr {
     float ABfx, ABfy, ABfz;  // A - B in FP32 (the FP32 kernels' horizontal step uses no FP64 instruction)
 };
 
+// Primitive-pair record of the Hermite-accumulator kernels: P, K (a + b)^-W with the prefactor K of PrimPair
+// and W = l_A + l_B, u = 2b, v = 2p, and the type of p in the exponent table.  Four 16-byte loads.
+struct alignas(16) HermPair {
+    double Px, Py, Pz;
+    double K;
+    double u, v;
+    int type, pad[3];
+};
+
+// What the Hermite-accumulator kernels read of a system: records (HermPair of pair t at t maxpp, sorted by
+// bound), their bounds in an array of their own (the screening loops read nothing else), and the exponent table
+// (nullptr: evaluate directly).
+struct HermView {
+    const HermPair* rec;
+    const float* B;
+    const double2* etab;
+    int ntype;
+};
+constexpr int kHermMaxTypes = 1448;  // 32 MB of exponent table
+
 struct EriArgs {
     const PairHdr* pairs;
     const void* prims64;  // PrimPair<double>[]
@@ -64,12 +84,13 @@ struct EriArgs {
     long long kstride;                // kets per field row of the ket table
     const PairHdr* bhdr;              // headers of the bra list in list order (bhdr[b] = pairs[bra[b]])
     const PairHdr* khdr;              // headers of the ket list in list order (khdr[k] = pairs[ket[k]])
+    HermView herm;
     int sort_work;                    // 1: each warp runs its window of quartets sorted by staircase length
 };
 
 struct SchwarzArgs {
     const PairHdr* pairs;
-    const void* prims64;  // PrimPair<double>[]
+    HermView herm;
     const int* ids;       // pair ids of one diagonal class
     int n;
     double* Q;            // [pair id] output bound
@@ -80,10 +101,9 @@ struct SchwarzArgs {
 
 // One molecule's view of one class in a batched build.
 struct MolClass {
-    const PairHdr* pairs;
-    const void* prims64;
-    const int* bra;
-    const int* ket;
+    const PairHdr* bhdr;  // headers of the bra and ket lists in list order
+    const PairHdr* khdr;
+    HermView herm;
     const long long* offsets;  // [n_bra + 1]
     int n_bra;
     int same;
@@ -107,6 +127,16 @@ struct BatchArgs {
 
 struct EriClassEntry {
     int X, Y, L;
+    // Hermite-accumulator kernels (the FP64 default): the thread kernel (nullptr: the class has none), the warp
+    // kernel (nullptr: none), its blocks per SM, operations per primitive and per contracted quartet
+    int prim_flops_h, cont_flops_h;
+    void (*launch_herm)(const EriArgs&, int grid, cudaStream_t, int lanes);
+    int herm_lanes;  // lanes per quartet of the thread kernel in small launches
+    void (*launch_hermw)(const EriArgs&, int grid, cudaStream_t, int nparts);
+    int (*prepare)();             // sets the kernels' shared-memory limits once per device
+    size_t (*local_bytes_h)();
+    int batch_warp;               // 1: the batched kernel is one warp per block
+    // Obara-Saika kernels: FP32, and FP64 with HF_OBARA_SAIKA
     int prim_flops;  // per primitive quartet (setup + Boys + VRR + accumulation)
     int cont_flops;  // per contracted quartet (HRR + digestion)
     void (*launch)(const EriArgs&, int use_f32, int grid, int block, cudaStream_t, int lanes);
@@ -119,16 +149,16 @@ struct EriClassEntry {
     void (*launch_rys)(const EriArgs&, int use_f32, int grid, int block, cudaStream_t, int lanes);
     int prim_flops_rys;       // per primitive quartet (setup + roots + 2D recurrences + accumulation)
     size_t (*local_bytes_rys)();
-    int rys_default;          // 1: FP64 launches use the Rys variant unless HF_OBARA_SAIKA is given
 };
 extern const EriClassEntry kEriClasses[kNumClasses];
 
-// Whether the FP64 launches of class ci take the Rys variant under these build flags: HF_RYS for every
-// class that has one, HF_OBARA_SAIKA for none, else the class's default.
-inline bool class_uses_rys(int ci, int flags)
+// Method of the FP64 launches of class ci under these build flags: Obara-Saika with HF_OBARA_SAIKA, Rys
+// quadrature with HF_RYS for the classes that have it, else Hermite accumulators.
+enum class Fp64Method { kHerm, kObaraSaika, kRys };
+inline Fp64Method fp64_method(int ci, int flags)
 {
-    if (!kEriClasses[ci].launch_rys || (flags & HF_OBARA_SAIKA)) return false;
-    return (flags & HF_RYS) || kEriClasses[ci].rys_default;
+    if (flags & HF_OBARA_SAIKA) return Fp64Method::kObaraSaika;
+    return (flags & HF_RYS) && kEriClasses[ci].launch_rys ? Fp64Method::kRys : Fp64Method::kHerm;
 }
 
 // Launches the ERI class kernels of one build: for every class and precision, the quartets
@@ -182,6 +212,30 @@ struct DevBuf {
     DevBuf& operator=(const DevBuf&) = delete;
 };
 
+// Exponent table over the distinct primitive exponents of one or several bases (HermView::etab); empty (tab.p
+// nullptr) when they give more than kHermMaxTypes sums.
+struct ExponentTable {
+    std::vector<double> exps;  // distinct, ascending
+    DevBuf tab, psum;
+    int ntype = 0;
+    void add(const hf_basis& b);
+    int build(cudaStream_t s);
+    HermView view(HermView h) const
+    {
+        h.etab = tab.as<double2>();
+        h.ntype = ntype;
+        return h;
+    }
+};
+
+// Status of hf_system_create's argument checks.
+int check_geometry_basis(const hf_geometry* g, const hf_basis* b, const hf_thresholds* th);
+
+// hf_system_create on a shared exponent table (nullptr: the system builds its own).  A shared table holds every
+// exponent of the basis and outlives the system.
+int create_system(hf_ctx* ctx, const hf_geometry* geom, const hf_basis* basis, const hf_thresholds* th,
+                  const ExponentTable* shared, hf_system** out);
+
 }  // namespace hf
 
 // ----------------------------------------------------------- C-ABI types --
@@ -211,6 +265,9 @@ struct hf_system {
     // pairs
     int n_pairs_all = 0, n_prim_pairs = 0;
     hf::DevBuf pairs, prims64, prims32, pair_class;
+    hf::DevBuf hrec, hB;          // HermPair records and bounds (HermView)
+    hf::ExponentTable etab;       // unless a batch's systems share one
+    hf::HermView herm{};
     int class_count[hf::kNumPairClasses] = {};
     hf::DevBuf class_ids[hf::kNumPairClasses];  // sorted significant pair ids
     double Qmax = 0.0;

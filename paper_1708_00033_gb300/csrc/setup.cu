@@ -135,7 +135,7 @@ __global__ void k_build_pairs(long long n_pairs, int maxpp, const int* __restric
                               const double* __restrict__ exps, const double* __restrict__ cn,
                               const double* __restrict__ xyz, PairHdr* __restrict__ pairs,
                               PrimPair<double>* __restrict__ p64, PrimPair<float>* __restrict__ p32,
-                              int* __restrict__ pclass)
+                              HermPair* __restrict__ hrec, const int* __restrict__ utype, int* __restrict__ pclass)
 {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n_pairs) return;
@@ -183,6 +183,18 @@ __global__ void k_build_pairs(long long n_pairs, int maxpp, const int* __restric
             r.oo2p = 0.5 * ip;
             r.B = 0.0f;  // set by the Schwarz pass; 0 never stops a primitive loop whose threshold is 0
             p64[t * maxpp + k] = r;
+            HermPair q;
+            q.Px = r.Px;
+            q.Py = r.Py;
+            q.Pz = r.Pz;
+            q.K = r.K;
+            for (int x = 0; x < la + lb; x++) q.K *= r.oo2p;
+            q.u = 2.0 * b;
+            q.v = 2.0 * p;
+            const int ta = utype[prim0[A] + ka], tb = utype[prim0[B] + kb];
+            q.type = max(ta, tb) * (max(ta, tb) + 1) / 2 + min(ta, tb);
+            q.pad[0] = q.pad[1] = q.pad[2] = 0;
+            hrec[t * maxpp + k] = q;
             PrimPair<float> f;
             f.p = (float)r.p;
             f.Px = (float)r.Px;
@@ -197,7 +209,6 @@ __global__ void k_build_pairs(long long n_pairs, int maxpp, const int* __restric
             p32[t * maxpp + k] = f;
         }
     }
-    (void)la;
 }
 
 __global__ void k_class_count(long long n, const int* __restrict__ pclass, unsigned long long* __restrict__ cnt)
@@ -291,26 +302,33 @@ int bitonic_sort_desc(double* key, int* val, int n, int n_pad, cudaStream_t s)
 // bound, largest first, so that the ERI loops can stop at the first
 // primitive quartet whose bound product falls below the primitive threshold.
 __global__ void k_sort_prims(long long n_pairs, const PairHdr* __restrict__ pairs, const double* __restrict__ Bprim,
-                             PrimPair<double>* __restrict__ p64, PrimPair<float>* __restrict__ p32)
+                             PrimPair<double>* __restrict__ p64, PrimPair<float>* __restrict__ p32,
+                             HermPair* __restrict__ hrec, float* __restrict__ hB)
 {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n_pairs) return;
     const int o = pairs[t].prim0, n = pairs[t].nprim;
     for (int k = 0; k < n; k++) {
+        hB[o + k] = (float)Bprim[o + k];
         p64[o + k].B = (float)Bprim[o + k];
         p32[o + k].B = (float)Bprim[o + k];
     }
     for (int i = 1; i < n; i++) {  // insertion sort, descending B
         const PrimPair<double> r = p64[o + i];
         const PrimPair<float> f = p32[o + i];
+        const HermPair h = hrec[o + i];
         int j = i - 1;
-        while (j >= 0 && p64[o + j].B < r.B) {
+        while (j >= 0 && hB[o + j] < r.B) {
             p64[o + j + 1] = p64[o + j];
             p32[o + j + 1] = p32[o + j];
+            hrec[o + j + 1] = hrec[o + j];
+            hB[o + j + 1] = hB[o + j];
             j--;
         }
         p64[o + j + 1] = r;
         p32[o + j + 1] = f;
+        hrec[o + j + 1] = h;
+        hB[o + j + 1] = r.B;
     }
 }
 
@@ -367,11 +385,28 @@ int launch_ket_table(int n, int maxpp, long long stride, const int* ids, const P
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-int launch_sort_prims(long long n_pairs, const PairHdr* pairs, const double* Bprim, void* p64, void* p32, cudaStream_t s)
+// Exponent table of the Hermite kernels (herm_exponents): entry (i, j) = 1/sqrt(p + q), 2 p q / (p + q) for the
+// exponent sums p = psum[i], q = psum[j].
+__global__ void k_exponent_table(int n, const double* __restrict__ psum, double2* __restrict__ tab)
+{
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= (long long)n * n) return;
+    const double p = psum[t / n], q = psum[t % n], s = p + q;
+    tab[t] = make_double2(1.0 / sqrt(s), 2.0 * p * q / s);
+}
+
+int launch_exponent_table(int n, const double* psum, double2* tab, cudaStream_t s)
+{
+    k_exponent_table<<<(unsigned)(((long long)n * n + 255) / 256), 256, 0, s>>>(n, psum, tab);
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+int launch_sort_prims(long long n_pairs, const PairHdr* pairs, const double* Bprim, void* p64, void* p32, HermPair* hrec,
+                      float* hB, cudaStream_t s)
 {
     if (n_pairs > 0)
         k_sort_prims<<<(unsigned)((n_pairs + 127) / 128), 128, 0, s>>>(n_pairs, pairs, Bprim, (PrimPair<double>*)p64,
-                                                                     (PrimPair<float>*)p32);
+                                                                     (PrimPair<float>*)p32, hrec, hB);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -521,12 +556,12 @@ int launch_comp_norm(int n_sh, const int* l, const int* bf0, double* out, cudaSt
 
 int launch_build_pairs(long long n_pairs, int maxpp, const int* l, const int* atom, const int* bf0, const int* nprim,
                        const int* prim0, const double* exps, const double* cn, const double* xyz, PairHdr* pairs,
-                       void* p64, void* p32, int* pclass, cudaStream_t s)
+                       void* p64, void* p32, HermPair* hrec, const int* utype, int* pclass, cudaStream_t s)
 {
     if (n_pairs == 0) return 0;
     k_build_pairs<<<(unsigned)((n_pairs + 127) / 128), 128, 0, s>>>(n_pairs, maxpp, l, atom, bf0, nprim, prim0, exps, cn,
                                                                   xyz, pairs, (PrimPair<double>*)p64,
-                                                                  (PrimPair<float>*)p32, pclass);
+                                                                  (PrimPair<float>*)p32, hrec, utype, pclass);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

@@ -12,7 +12,7 @@ int launch_shell_coef(int n_sh, const int* l, const int* nprim, const int* prim0
 int launch_comp_norm(int n_sh, const int* l, const int* bf0, double* out, cudaStream_t s);
 int launch_build_pairs(long long n_pairs, int maxpp, const int* l, const int* atom, const int* bf0, const int* nprim,
                        const int* prim0, const double* exps, const double* cn, const double* xyz, PairHdr* pairs,
-                       void* p64, void* p32, int* pclass, cudaStream_t s);
+                       void* p64, void* p32, HermPair* hrec, const int* utype, int* pclass, cudaStream_t s);
 int launch_class_count(long long n, const int* pclass, unsigned long long* cnt, cudaStream_t s);
 int launch_class_scatter_all(long long n, const int* pclass, int X, unsigned* cursor, int* ids, cudaStream_t s);
 int launch_copy_q(long long n, const double* Q, PairHdr* pairs, unsigned long long* qmax_bits, cudaStream_t s);
@@ -22,7 +22,9 @@ int bitonic_sort_desc(double* key, int* val, int n, int n_pad, cudaStream_t s);
 int launch_gather_headers(int n, const int* ids, const PairHdr* pairs, PairHdr* out, cudaStream_t s);
 int launch_ket_table(int n, int maxpp, long long stride, const int* ids, const PairHdr* pairs, const void* p64,
                      const void* p32, double* t64, float* t32, float* tB, cudaStream_t s);
-int launch_sort_prims(long long n_pairs, const PairHdr* pairs, const double* Bprim, void* p64, void* p32, cudaStream_t s);
+int launch_sort_prims(long long n_pairs, const PairHdr* pairs, const double* Bprim, void* p64, void* p32, HermPair* hrec,
+                      float* hB, cudaStream_t s);
+int launch_exponent_table(int n, const double* psum, double2* tab, cudaStream_t s);
 int launch_scan(int n, const long long* in, long long* out, cudaStream_t s);
 int launch_sig_scatter(long long n_pairs, long long n_seg, const int* pclass, const double* Q,
                        const unsigned long long* qmax_bits, double tau, const size_t* seg_host, unsigned* cursor,
