@@ -264,6 +264,34 @@ struct Arena {
     }
 };
 
+// The context's side streams between an event recorded on its stream and one it waits for; the destructor joins
+// what an early return left running, which still uses the caller's buffers.
+struct SideStreams {
+    hf_ctx* ctx;
+    bool open = false;
+    explicit SideStreams(hf_ctx* c) : ctx(c) {}
+    int fork()
+    {
+        HF_CUDA(cudaEventRecord(ctx->fork, ctx->stream));
+        open = true;
+        for (auto& s : ctx->side) HF_CUDA(cudaStreamWaitEvent(s, ctx->fork, 0));
+        return HF_OK;
+    }
+    int join()
+    {
+        if (!open) return HF_OK;
+        open = false;
+        cudaError_t err = cudaSuccess;
+        for (int i = 0; i < kSideStreams; i++) {
+            const cudaError_t e1 = cudaEventRecord(ctx->join[i], ctx->side[i]);
+            const cudaError_t e2 = cudaStreamWaitEvent(ctx->stream, ctx->join[i], 0);
+            if (err == cudaSuccess) err = e1 != cudaSuccess ? e1 : e2;
+        }
+        return err == cudaSuccess ? HF_OK : cuda_status(err, "joining the side streams");
+    }
+    ~SideStreams() { join(); }
+};
+
 static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* basis, const ExponentTable* shared)
 {
     hf_ctx* ctx = S->ctx;
@@ -378,11 +406,6 @@ static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* b
     KCHK(launch_shell_coef(ns, S->sh_l.as<int>(), S->sh_nprim.as<int>(), S->sh_prim0.as<int>(), S->sh_exp.as<double>(),
                            coef_in.as<double>(), S->sh_coef.as<double>(), st));
     KCHK(launch_comp_norm(ns, S->sh_l.as<int>(), S->sh_bf0.as<int>(), S->comp_norm.as<double>(), st));
-    KCHK(launch_one_electron(ns, na, nbf, S->sh_l.as<int>(), S->sh_atom.as<int>(), S->sh_bf0.as<int>(),
-                             S->sh_nprim.as<int>(), S->sh_prim0.as<int>(), S->sh_exp.as<double>(),
-                             S->sh_coef.as<double>(), S->atom_xyz.as<double>(), S->atom_Z.as<double>(),
-                             S->comp_norm.as<double>(), ctx->boys64.as<double>(), S->S.as<double>(),
-                             S->H.as<double>(), st));
     KCHK(launch_nuclear_repulsion(na, S->atom_xyz.as<double>(), S->atom_Z.as<double>(), S->Ebuf.as<double>() + 300,
                                   st));
     KCHK(launch_build_pairs(npairs, X.maxpp, S->sh_l.as<int>(), S->sh_atom.as<int>(), S->sh_bf0.as<int>(),
@@ -430,21 +453,35 @@ static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* b
     // --------------------------------------------------- Schwarz bounds
     HF_CUDA(cudaMemsetAsync(X.Qall.p, 0, sizeof(double) * npairs, st));
     HF_CUDA(cudaMemsetAsync(X.Bprim.p, 0, sizeof(double) * npairs * X.maxpp, st));
-    for (int c = 0; c < kNumPairClasses; c++) {
-        if (!cnt_all[c]) continue;
-        int* ids = ids_all.as<int>() + base_all[c];
-        KCHK(launch_class_scatter_all(npairs, S->pair_class.as<int>(), c, (unsigned*)(cnt_dev + 8 + c), ids, st));
-        SchwarzArgs sa;
-        sa.pairs = S->pairs.as<PairHdr>();
-        sa.herm = S->herm;
-        sa.ids = ids;
-        sa.n = (int)cnt_all[c];
-        sa.Q = X.Qall.as<double>();
-        sa.boys64 = ctx->boys64.as<double>();
-        sa.Bprim = X.Bprim.as<double>();
-        sa.items = X.maxpp + 1;
-        kEriClasses[class_index(c, c)].launch_schwarz(sa, kEriThreads, st);
-        HF_CUDA(cudaGetLastError());
+    for (int c = 0; c < kNumPairClasses; c++)
+        if (cnt_all[c])
+            KCHK(launch_class_scatter_all(npairs, S->pair_class.as<int>(), c, (unsigned*)(cnt_dev + 8 + c),
+                                          ids_all.as<int>() + base_all[c], st));
+    // bounds and one-electron blocks of the classes run concurrently: each lasts as long as its longest pair
+    {
+        SideStreams side(ctx);
+        TRY(side.fork());
+        for (int c = 0; c < kNumPairClasses; c++) {
+            if (!cnt_all[c]) continue;
+            int* ids = ids_all.as<int>() + base_all[c];
+            SchwarzArgs sa;
+            sa.pairs = S->pairs.as<PairHdr>();
+            sa.herm = S->herm;
+            sa.ids = ids;
+            sa.n = (int)cnt_all[c];
+            sa.Q = X.Qall.as<double>();
+            sa.boys64 = ctx->boys64.as<double>();
+            sa.Bprim = X.Bprim.as<double>();
+            sa.items = X.maxpp + 1;
+            kEriClasses[class_index(c, c)].launch_schwarz(sa, kEriThreads, ctx->side[c]);
+            HF_CUDA(cudaGetLastError());
+            OneEArgs oa{S->pairs.as<PairHdr>(), ids, (int)cnt_all[c], na, nbf, S->sh_nprim.as<int>(),
+                        S->sh_prim0.as<int>(), S->sh_exp.as<double>(), S->sh_coef.as<double>(),
+                        S->atom_xyz.as<double>(), S->atom_Z.as<double>(), S->comp_norm.as<double>(),
+                        ctx->boys64.as<double>(), S->herm, S->S.as<double>(), S->H.as<double>()};
+            KCHK(launch_one_electron_class(c, oa, ctx->side[(c + 3) % kSideStreams]));
+        }
+        TRY(side.join());
     }
     KCHK(launch_sort_prims(npairs, S->pairs.as<PairHdr>(), X.Bprim.as<double>(), S->prims64.p, S->prims32.p,
                            S->hrec.as<HermPair>(), S->hB.as<float>(), st));
@@ -456,33 +493,36 @@ static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* b
     const double tau = S->th.schwarz_tau;
     KCHK(launch_sig_scatter(npairs, (long long)seg[kNumPairClasses], S->pair_class.as<int>(), X.Qall.as<double>(),
                             qbits_dev, tau, seg, nsig_dev, key.as<double>(), val.as<int>(), st));
+    SideStreams sorts(ctx);
+    TRY(sorts.fork());
     for (int c = 0; c < kNumPairClasses; c++) {
         if (!npad[c]) continue;
-        KCHK(bitonic_sort_desc(key.as<double>() + seg[c], val.as<int>() + seg[c], (int)npad[c], (int)npad[c], st));
+        KCHK(bitonic_sort_desc(key.as<double>() + seg[c], val.as<int>() + seg[c], (int)npad[c], (int)npad[c],
+                               ctx->side[c]));
         S->class_ids[c].view(val.as<int>() + seg[c], sizeof(int) * npad[c]);
         X.class_q[c].view(key.as<double>() + seg[c], sizeof(double) * npad[c]);
     }
 
+    TRY(sorts.join());
+
     // ------------------------------------------------- quartet schedule
     S->quartets_total = 0;
+    QuartetSchedule qs{};
+    qs.tau = tau;
+    qs.cutoff = S->th.fp32_cutoff;
+    qs.totals = totals_dev;
     for (int ci = 0; ci < kNumClasses; ci++) {
         const int Xc = kEriClasses[ci].X, Yc = kEriClasses[ci].Y;
         auto& pl = S->plan[ci];
         pl.n_unscreened = (Xc == Yc) ? (long long)cnt_all[Xc] * (cnt_all[Xc] + 1) / 2
                                      : (long long)cnt_all[Xc] * (long long)cnt_all[Yc];
         S->quartets_total += pl.n_unscreened;
-        const int cap = (int)cnt_all[Xc];
-        if (!cap || !cnt_all[Yc]) continue;
-        KCHK(launch_ket_counts_dev(cap, nsig_dev + Xc, X.class_q[Xc].as<double>(), nsig_dev + Yc,
-                                   X.class_q[Yc].as<double>(), Xc == Yc, tau, S->th.fp32_cutoff, c64[ci].as<long long>(),
-                                   c32[ci].as<long long>(), pl.kstart32.as<int>(), st));
-        KCHK(launch_scan(cap, c64[ci].as<long long>(), pl.offsets64.as<long long>(), st));
-        KCHK(launch_scan(cap, c32[ci].as<long long>(), pl.offsets32.as<long long>(), st));
-        HF_CUDA(cudaMemcpyAsync(totals_dev + 2 * ci, pl.offsets64.as<long long>() + cap, sizeof(long long),
-                                cudaMemcpyDeviceToDevice, st));
-        HF_CUDA(cudaMemcpyAsync(totals_dev + 2 * ci + 1, pl.offsets32.as<long long>() + cap, sizeof(long long),
-                                cudaMemcpyDeviceToDevice, st));
+        if (!cnt_all[Xc] || !cnt_all[Yc]) continue;
+        qs.c[ci] = {(int)cnt_all[Xc], Xc == Yc, nsig_dev + Xc, nsig_dev + Yc, X.class_q[Xc].as<double>(),
+                    X.class_q[Yc].as<double>(), c64[ci].as<long long>(), c32[ci].as<long long>(),
+                    pl.offsets64.as<long long>(), pl.offsets32.as<long long>(), pl.kstart32.as<int>()};
     }
+    KCHK(launch_quartet_schedule(qs, st));
     HF_CUDA(cudaMemcpyAsync(enn_dev, S->Ebuf.as<double>() + 300, sizeof(double), cudaMemcpyDeviceToDevice, st));
     HF_CUDA(cudaMemcpyAsync(enn_dev + 1, qbits_dev, sizeof(double), cudaMemcpyDeviceToDevice, st));
     unsigned char rbh[512];
@@ -497,36 +537,42 @@ static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* b
         S->plan[ci].n64 = totals_h[2 * ci];
         S->plan[ci].n32 = totals_h[2 * ci + 1];
     }
-    // ket tables (field-major copies of each class's records in class-list order)
+    // ket tables (field-major copies of each class's records in class-list order), headers in list order, and
+    // bra lookup tables: one allocation, whose sizes follow from the counts just read
+    Arena a4;
+    const size_t rows = (size_t)X.maxpp;
     for (int c = 0; c < kNumPairClasses; c++) {
         const int n = S->class_count[c];
         if (n <= 0) continue;
-        const long long stride = ((long long)n + 31) / 32 * 32;
-        S->ket_stride[c] = stride;
-        const size_t rows = (size_t)X.maxpp;
-        TRY(S->ket_tab[c].alloc(rows * stride * (9 * sizeof(double) + 9 * sizeof(float) + sizeof(float))));
+        S->ket_stride[c] = ((long long)n + 31) / 32 * 32;
+        a4.add(S->ket_tab[c], rows * S->ket_stride[c] * (9 * sizeof(double) + 9 * sizeof(float) + sizeof(float)));
+        a4.add(S->class_hdr[c], sizeof(PairHdr) * (size_t)n);
+    }
+    for (auto& pl : S->plan) {
+        if (pl.n64 > 0) a4.add(pl.chunk64, sizeof(int) * chunk_entries(pl.n64));
+        if (pl.n32 > 0) a4.add(pl.chunk32, sizeof(int) * chunk_entries(pl.n32));
+    }
+    TRY(a4.commit(X.arena_tab));
+    for (int c = 0; c < kNumPairClasses; c++) {
+        const int n = S->class_count[c];
+        if (n <= 0) continue;
+        const long long stride = S->ket_stride[c];
         double* t64 = S->ket_tab[c].as<double>();
         float* t32 = (float*)(t64 + 9 * rows * stride);
         float* tB = t32 + 9 * rows * stride;
         KCHK(launch_ket_table(n, X.maxpp, stride, S->class_ids[c].as<int>(), S->pairs.as<PairHdr>(), S->prims64.p,
                               S->prims32.p, t64, t32, tB, st));
-        TRY(S->class_hdr[c].alloc(sizeof(PairHdr) * (size_t)n));
         KCHK(launch_gather_headers(n, S->class_ids[c].as<int>(), S->pairs.as<PairHdr>(), S->class_hdr[c].as<PairHdr>(),
                                    st));
     }
-    // bra lookup tables (their sizes follow from the quartet totals)
+    ChunkTables ct{};
     for (int ci = 0; ci < kNumClasses; ci++) {
         auto& pl = S->plan[ci];
         const int nb = S->class_count[kEriClasses[ci].X];
-        if (pl.n64 > 0) {
-            TRY(pl.chunk64.alloc(sizeof(int) * chunk_entries(pl.n64)));
-            KCHK(launch_chunk_bra(nb, pl.offsets64.as<long long>(), pl.n64, pl.chunk64.as<int>(), st));
-        }
-        if (pl.n32 > 0) {
-            TRY(pl.chunk32.alloc(sizeof(int) * chunk_entries(pl.n32)));
-            KCHK(launch_chunk_bra(nb, pl.offsets32.as<long long>(), pl.n32, pl.chunk32.as<int>(), st));
-        }
+        if (pl.n64 > 0) ct.t[ct.n++] = {nb, pl.offsets64.as<long long>(), pl.n64, chunk_entries(pl.n64), pl.chunk64.as<int>()};
+        if (pl.n32 > 0) ct.t[ct.n++] = {nb, pl.offsets32.as<long long>(), pl.n32, chunk_entries(pl.n32), pl.chunk32.as<int>()};
     }
+    KCHK(launch_chunk_bra(ct, st));
     HF_CUDA(cudaGetLastError());
     return HF_OK;
 }

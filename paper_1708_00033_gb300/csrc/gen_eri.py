@@ -831,6 +831,15 @@ def main(outdir):
         if not os.path.exists(path) or open(path).read() != text:
             with open(path, "w") as fh:
                 fh.write(text)
+    lines = [HEADER.replace("eri_common.cuh", "onee_herm.cuh").replace("One shell-quartet class per file", "One-electron kernels, one per pair class")]
+    lines += [gen_herm.gen_onee(la, lb) for la, lb in PAIR_CLASSES]
+    lines.append("int launch_one_electron_class(int X, const OneEArgs& a, cudaStream_t s)\n{\n    switch (X) {")
+    lines += [f"        case {x}: return launch_one_electron_{la}{lb}(a, s);" for x, (la, lb) in enumerate(PAIR_CLASSES)]
+    lines += ["    }", "    return -1;", "}", FOOTER]
+    path, text = os.path.join(outdir, "onee_pairs.cu"), "\n".join(lines)
+    if not os.path.exists(path) or open(path).read() != text:
+        with open(path, "w") as fh:
+            fh.write(text)
     # dispatch table
     lines = ['// Generated by gen_eri.py: do not edit.', '#include "eri_common.cuh"', "", "namespace hf {"]
     for info in infos:

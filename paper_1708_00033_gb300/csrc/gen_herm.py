@@ -417,3 +417,47 @@ def gen_warp(name, la, lb, lc, ld):
     co.n += k3.n * nab + 12 * nab * ncd
     o.append("};")
     return "\n".join(o) + "\n", po.n, co.n
+
+
+def gen_onee(la, lb):
+    """Traits of the one-electron kernel of a pair class (one_electron_pair in onee_herm.cuh): nuclear attraction
+    with the same Hermite accumulators, a point charge in the ket's place."""
+    L = la + lb
+    hs, sc, its = hermites(L), list(scalings(la, lb)), items(la, lb)
+    hidx = {t: i for i, t in enumerate(hs)}
+    ops = Ops()
+    o = [f"struct OneE_{la}{lb} {{",
+         f"    static constexpr int LA = {la}, LB = {lb}, NR = {len(hs)}, NI = {len(its)};",
+         "    // RS += Z R_N(P - C)",
+         "    static __device__ __forceinline__ void nucleus(const HermPair& bp, double Cx, double Cy, double Cz, double Z,"
+         " const double* __restrict__ boys_tab, double (&RS)[NR])",
+         "    {",
+         "        const double Dx = Cx - bp.Px, Dy = Cy - bp.Py, Dz = Cz - bp.Pz;",
+         f"        double F[{L + 1}];",
+         f"        boys_eval_2t<{L}>(bp.v * (Dx * Dx + Dy * Dy + Dz * Dz), boys_tab, F);",
+         "        double zp = Z;"]
+    for m in range(L + 1):
+        if m:
+            o.append("        zp *= bp.v;")
+        o.append(f"        const double g{m} = zp * F[{m}];")
+    lines, rname = r_lines(L, ops)
+    o += ["        " + l for l in lines]
+    o += [f"        RS[{i}] += {rname(t)};" for i, t in enumerate(hs)]
+    o += ["    }", "    // acc += pf sigma RS_N of every scaling and order",
+          "    static __device__ __forceinline__ void scale(const HermPair& bp, double pf, const double (&RS)[NR], double (&acc)[NI])",
+          "    {"]
+    lines, names = scale_lines(la, lb, "bp", "ub", ops)
+    o += ["        " + l for l in lines]
+    for i, n in enumerate(names):
+        o.append(f"        const double sb{i} = pf" + (f" * {n};" if n else ";"))
+    o += [f"        acc[{x}] = fma(sb{sc.index((k, s))}, RS[{hidx[t]}], acc[{x}]);" for x, (k, s, t) in enumerate(its)]
+    o += ["    }", "    // (a|b) from the accumulators",
+          "    static __device__ __forceinline__ void finish(const double (&acc)[NI], double ABx, double ABy, double ABz, double* __restrict__ V)",
+          "    {"]
+    pos = {it: x for x, it in enumerate(its)}
+    lines, out = transform(la, lb, lambda k, s, t: f"acc[{pos[(k, s, t)]}]", "AB", False, ops, "x")
+    l2, ab = hrr(la, lb, lambda e: out[e], "AB", ops, "p")
+    o += ["        " + l for l in lines + l2]
+    o += [f"        V[{i}] = {ab[k]};" for i, k in enumerate((a, b) for a in CART[la] for b in CART[lb])]
+    o += ["    }", "};", f"ONEE_KERNEL({la}, {lb})", ""]
+    return "\n".join(o)

@@ -99,6 +99,26 @@ struct SchwarzArgs {
     int items;            // threads per pair: 1 + the largest primitive-pair count
 };
 
+// One-electron matrices of one pair class (onee_herm.cuh).
+struct OneEArgs {
+    const PairHdr* pairs;
+    const int* ids;  // pair ids of the class
+    int n, n_atoms, N;
+    const int* nprim;
+    const int* prim0;
+    const double* exps;
+    const double* cn;
+    const double* xyz;
+    const double* Z;
+    const double* comp_norm;
+    const double* boys64;
+    HermView herm;
+    double* S;
+    double* H;
+};
+
+int launch_one_electron_class(int X, const OneEArgs& a, cudaStream_t s);
+
 // One molecule's view of one class in a batched build.
 struct MolClass {
     const PairHdr* bhdr;  // headers of the bra and ket lists in list order
@@ -284,7 +304,7 @@ struct hf_system {
     // scratch
     hf::DevBuf class_q[hf::kNumPairClasses];  // sorted bounds of class_ids
     hf::DevBuf Qall, counts, staging_P, staging_out, bad, Bprim, prim_count;
-    hf::DevBuf arena_in, arena_mat, arena_sched;  // owners of the views above
+    hf::DevBuf arena_in, arena_mat, arena_sched, arena_tab;  // owners of the views above
     hf::DevBuf dsh;                                // density block maxima for density-weighted screening
     // ket tables: per pair class, the significant pairs' primitive-pair records in class-list order and
     // field-major (9 maxpp rows of FP64 fields, 9 maxpp rows of FP32 fields, maxpp rows of bounds)

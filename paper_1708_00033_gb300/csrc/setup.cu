@@ -247,20 +247,6 @@ __global__ void k_max_q(long long n, const double* __restrict__ Q, unsigned long
     if (threadIdx.x == 0) atomicMax(out, (unsigned long long)__double_as_longlong(sm[0]));
 }
 
-// significant pairs of class X: Q * Qmax >= tau (tau = 0 keeps all)
-__global__ void k_class_scatter_sig(long long n, const int* __restrict__ pclass, const double* __restrict__ Q, int X,
-                                    double qmax, double tau, unsigned* __restrict__ cursor, double* __restrict__ key,
-                                    int* __restrict__ val)
-{
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n || pclass[t] != X) return;
-    const double q = Q[t];
-    if (tau > 0.0 && !(q * qmax >= tau)) return;
-    const unsigned pos = atomicAdd(cursor, 1u);
-    key[pos] = q;
-    val[pos] = (int)t;
-}
-
 __global__ void k_fill_pad(int from, int n_pad, double* key, int* val)
 {
     const int t = from + blockIdx.x * blockDim.x + threadIdx.x;
@@ -289,12 +275,55 @@ __global__ void k_bitonic_step(double* __restrict__ key, int* __restrict__ val, 
     }
 }
 
+// The same network's steps with distance below kSortTile inside tiles of kSortTile elements in shared memory: whole
+// stages k <= kSortTile (k_first == 2), or the end j < kSortTile of stage k_first.  One launch in place of 66
+// (first) and 11 (each later stage).
+constexpr unsigned kSortTile = 2048;
+__global__ void __launch_bounds__(1024) k_bitonic_tile(double* __restrict__ key, int* __restrict__ val, unsigned n_pad,
+                                                       unsigned k_first, unsigned k_last)
+{
+    __shared__ double sk[kSortTile];
+    __shared__ int sv[kSortTile];
+    const unsigned base = blockIdx.x * kSortTile, m = min(kSortTile, n_pad);
+    for (unsigned i = threadIdx.x; i < m; i += 1024) {
+        sk[i] = key[base + i];
+        sv[i] = val[base + i];
+    }
+    __syncthreads();
+    for (unsigned k = k_first; k <= k_last; k <<= 1)
+        for (unsigned j = min(k, m) >> 1; j > 0; j >>= 1) {
+            for (unsigned t = threadIdx.x; t < m / 2; t += 1024) {
+                const unsigned i = 2 * t - (t & (j - 1)), l = i + j;
+                const double ki = sk[i], kl = sk[l];
+                const int vi = sv[i], vl = sv[l];
+                const bool l_first = (kl > ki) || (kl == ki && vl < vi);
+                if (((base + i) & k) == 0 ? l_first : !l_first) {
+                    sk[i] = kl;
+                    sk[l] = ki;
+                    sv[i] = vl;
+                    sv[l] = vi;
+                }
+            }
+            __syncthreads();
+        }
+    for (unsigned i = threadIdx.x; i < m; i += 1024) {
+        key[base + i] = sk[i];
+        val[base + i] = sv[i];
+    }
+}
+
 int bitonic_sort_desc(double* key, int* val, int n, int n_pad, cudaStream_t s)
 {
     if (n_pad > n) k_fill_pad<<<(n_pad - n + 255) / 256, 256, 0, s>>>(n, n_pad, key, val);
-    for (unsigned k = 2; k <= (unsigned)n_pad; k <<= 1)
-        for (unsigned j = k >> 1; j > 0; j >>= 1)
-            k_bitonic_step<<<(n_pad + 255) / 256, 256, 0, s>>>(key, val, (unsigned)n_pad, j, k);
+    const unsigned np = (unsigned)n_pad;
+    if (np < 2) return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    const unsigned tiles = (np + kSortTile - 1) / kSortTile;
+    k_bitonic_tile<<<tiles, 1024, 0, s>>>(key, val, np, 2, np < kSortTile ? np : kSortTile);
+    for (unsigned k = 2 * kSortTile; k <= np; k <<= 1) {
+        for (unsigned j = k >> 1; j >= kSortTile; j >>= 1)
+            k_bitonic_step<<<(np + 255) / 256, 256, 0, s>>>(key, val, np, j, k);
+        k_bitonic_tile<<<tiles, 1024, 0, s>>>(key, val, np, k, k);
+    }
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -411,30 +440,55 @@ int launch_sort_prims(long long n_pairs, const PairHdr* pairs, const double* Bpr
 }
 
 // ------------------------------------------------------- quartet schedule --
-// exclusive scan of n counts into out[0..n] (single block, chunked)
-__global__ void k_scan(int n, const long long* __restrict__ in, long long* __restrict__ out)
+// Exclusive prefix sums out[0..n] of the counts, one block per (class, part): each thread sums its own run of
+// the chunk, the warps' sums are scanned with shuffles.  42 arrays, one launch (they took 42, and as many copies of
+// the totals).
+__global__ void __launch_bounds__(1024) k_scan_all(const QuartetSchedule q)
 {
-    __shared__ long long sm[1024];
-    __shared__ long long carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int base = 0; base < n; base += blockDim.x) {
-        const int i = base + threadIdx.x;
-        const long long v = i < n ? in[i] : 0;
-        sm[threadIdx.x] = v;
-        __syncthreads();
-        for (int off = 1; off < (int)blockDim.x; off <<= 1) {
-            const long long add = threadIdx.x >= (unsigned)off ? sm[threadIdx.x - off] : 0;
-            __syncthreads();
-            sm[threadIdx.x] += add;
-            __syncthreads();
+    const ClassCounts& c = q.c[blockIdx.x >> 1];
+    const bool part32 = blockIdx.x & 1;
+    const int n = c.cap;
+    if (n == 0) return;
+    const long long* const in = part32 ? c.c32 : c.c64;
+    long long* const out = part32 ? c.off32 : c.off64;
+    __shared__ long long wsum[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    long long carry = 0;
+    for (int base = 0; base < n; base += 4096) {
+        long long v[4], sum = 0;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int i = base + 4 * threadIdx.x + k;
+            v[k] = i < n ? in[i] : 0;
+            sum += v[k];
         }
-        if (i < n) out[i] = carry + sm[threadIdx.x] - v;
+        long long x = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wsum[warp] = x;
         __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) carry += sm[threadIdx.x];
+        long long before = 0, all = 0;
+        for (int w = 0; w < 32; w++) {
+            if (w < warp) before += wsum[w];
+            all += wsum[w];
+        }
+        long long e = carry + before + x - sum;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int i = base + 4 * threadIdx.x + k;
+            if (i < n) out[i] = e;
+            e += v[k];
+        }
+        carry += all;
         __syncthreads();
     }
-    if (threadIdx.x == 0) out[n] = carry;
+    if (threadIdx.x == 0) {
+        out[n] = carry;
+        q.totals[blockIdx.x] = carry;
+    }
 }
 
 // --------------------------------------------- all-class scatter and counts --
@@ -486,14 +540,16 @@ int launch_sig_scatter(long long n_pairs, long long n_seg, const int* pclass, co
 // prefix; when X == Y only kets k <= b are unique.  The prefix splits into an FP64 head
 // (Q_b Q_k >= cutoff) and an FP32 tail.  The list lengths are read on the device (entries
 // b >= n_bra get zero counts), so the schedule needs no host round trip.
-__global__ void k_ket_counts_dev(int cap, const unsigned* __restrict__ n_bra_p, const double* __restrict__ qb,
-                                 const unsigned* __restrict__ n_ket_p, const double* __restrict__ qk, int same,
-                                 double tau, double cutoff, long long* __restrict__ c64, long long* __restrict__ c32,
-                                 int* __restrict__ kstart32)
+__global__ void k_ket_counts(const QuartetSchedule q)
 {
+    const ClassCounts& c = q.c[blockIdx.y];
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= cap) return;
-    const int n_bra = (int)*n_bra_p, n_ket = (int)*n_ket_p;
+    if (b >= c.cap) return;
+    const int n_bra = (int)*c.n_bra, n_ket = (int)*c.n_ket;
+    const double *qb = c.qb, *qk = c.qk, tau = q.tau, cutoff = q.cutoff;
+    long long *c64 = c.c64, *c32 = c.c32;
+    int* const kstart32 = c.kstart32;
+    const int same = c.same;
     if (b >= n_bra || n_ket == 0) {
         c64[b] = 0;
         c32[b] = 0;
@@ -531,13 +587,13 @@ __global__ void k_ket_counts_dev(int cap, const unsigned* __restrict__ n_bra_p, 
     kstart32[b] = n64;
 }
 
-int launch_ket_counts_dev(int cap, const unsigned* n_bra, const double* qb, const unsigned* n_ket, const double* qk,
-                          int same, double tau, double cutoff, long long* c64, long long* c32, int* kstart32,
-                          cudaStream_t s)
+int launch_quartet_schedule(const QuartetSchedule& q, cudaStream_t s)
 {
-    if (cap > 0)
-        k_ket_counts_dev<<<(cap + 255) / 256, 256, 0, s>>>(cap, n_bra, qb, n_ket, qk, same, tau, cutoff, c64, c32,
-                                                            kstart32);
+    int cap = 0;
+    for (const ClassCounts& c : q.c) cap = c.cap > cap ? c.cap : cap;
+    if (cap == 0) return 0;
+    k_ket_counts<<<dim3((cap + 255) / 256, kNumClasses), 256, 0, s>>>(q);
+    k_scan_all<<<2 * kNumClasses, 1024, 0, s>>>(q);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -586,37 +642,23 @@ int launch_copy_q(long long n, const double* Q, PairHdr* pairs, unsigned long lo
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-int launch_class_scatter_sig(long long n, const int* pclass, const double* Q, int X, double qmax, double tau,
-                             unsigned* cursor, double* key, int* val, cudaStream_t s)
-{
-    if (n > 0)
-        k_class_scatter_sig<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, pclass, Q, X, qmax, tau, cursor, key, val);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
-}
-
-int launch_scan(int n, const long long* in, long long* out, cudaStream_t s)
-{
-    k_scan<<<1, 1024, 0, s>>>(n, in, out);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
-}
 
 // Bra lookup table of one class and precision: entry c = bra of quartet min(c << kChunkShift, n - 1),
 // c = 0 .. ((n - 1) >> kChunkShift) + 1, so that quartet q's bra lies in [t[q >> S], t[(q >> S) + 1]].
-__global__ void k_chunk_bra(int n_bra, const long long* __restrict__ off, long long n, long long n_entries,
-                            int* __restrict__ out)
+__global__ void k_chunk_bra(const ChunkTables a)
 {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n_entries) return;
-    const long long q = min(c << kChunkShift, n - 1);
-    out[c] = find_bra(off, n_bra, q);
+    const ChunkTable& t = a.t[blockIdx.y];
+    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < t.entries; c += (long long)gridDim.x * blockDim.x)
+        t.out[c] = find_bra(t.off, t.n_bra, min(c << kChunkShift, t.n - 1));
 }
 
 long long chunk_entries(long long n) { return n > 0 ? ((n - 1) >> kChunkShift) + 2 : 0; }
 
-int launch_chunk_bra(int n_bra, const long long* off, long long n, int* out, cudaStream_t s)
+int launch_chunk_bra(const ChunkTables& c, cudaStream_t s)
 {
-    const long long e = chunk_entries(n);
-    if (e > 0) k_chunk_bra<<<(unsigned)((e + 255) / 256), 256, 0, s>>>(n_bra, off, n, e, out);
+    long long most = 0;
+    for (int i = 0; i < c.n; i++) most = c.t[i].entries > most ? c.t[i].entries : most;
+    if (most > 0) k_chunk_bra<<<dim3((unsigned)min((most + 255) / 256, 1024LL), c.n), 256, 0, s>>>(c);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

@@ -16,8 +16,6 @@ int launch_build_pairs(long long n_pairs, int maxpp, const int* l, const int* at
 int launch_class_count(long long n, const int* pclass, unsigned long long* cnt, cudaStream_t s);
 int launch_class_scatter_all(long long n, const int* pclass, int X, unsigned* cursor, int* ids, cudaStream_t s);
 int launch_copy_q(long long n, const double* Q, PairHdr* pairs, unsigned long long* qmax_bits, cudaStream_t s);
-int launch_class_scatter_sig(long long n, const int* pclass, const double* Q, int X, double qmax, double tau,
-                             unsigned* cursor, double* key, int* val, cudaStream_t s);
 int bitonic_sort_desc(double* key, int* val, int n, int n_pad, cudaStream_t s);
 int launch_gather_headers(int n, const int* ids, const PairHdr* pairs, PairHdr* out, cudaStream_t s);
 int launch_ket_table(int n, int maxpp, long long stride, const int* ids, const PairHdr* pairs, const void* p64,
@@ -25,24 +23,41 @@ int launch_ket_table(int n, int maxpp, long long stride, const int* ids, const P
 int launch_sort_prims(long long n_pairs, const PairHdr* pairs, const double* Bprim, void* p64, void* p32, HermPair* hrec,
                       float* hB, cudaStream_t s);
 int launch_exponent_table(int n, const double* psum, double2* tab, cudaStream_t s);
-int launch_scan(int n, const long long* in, long long* out, cudaStream_t s);
+// Quartet schedule of every class in two launches: ket counts per bra (FP64 and FP32 part) and their exclusive
+// prefix sums, whose totals go to `totals`[2 class + part].
+struct ClassCounts {
+    int cap, same;  // cap: bras of the class list before screening (0: the class is empty)
+    const unsigned *n_bra, *n_ket;
+    const double *qb, *qk;
+    long long *c64, *c32, *off64, *off32;
+    int* kstart32;
+};
+struct QuartetSchedule {
+    ClassCounts c[kNumClasses];
+    double tau, cutoff;
+    long long* totals;
+};
+int launch_quartet_schedule(const QuartetSchedule& q, cudaStream_t s);
 int launch_sig_scatter(long long n_pairs, long long n_seg, const int* pclass, const double* Q,
                        const unsigned long long* qmax_bits, double tau, const size_t* seg_host, unsigned* cursor,
                        double* key, int* val, cudaStream_t s);
-int launch_ket_counts_dev(int cap, const unsigned* n_bra, const double* qb, const unsigned* n_ket, const double* qk,
-                          int same, double tau, double cutoff, long long* c64, long long* c32, int* kstart32,
-                          cudaStream_t s);
 
-// one-electron matrices (raw component normalisation; comp_norm applied inside)
-int launch_one_electron(int n_sh, int n_atoms, int N, const int* l, const int* atom, const int* bf0,
-                        const int* nprim, const int* prim0, const double* exps, const double* cn,
-                        const double* xyz, const double* Z, const double* comp_norm, const double* boys64,
-                        double* S, double* H, cudaStream_t s);
 int launch_nuclear_repulsion(int n_atoms, const double* xyz, const double* Z, double* out, cudaStream_t s);
 
 // Fock assembly
 long long chunk_entries(long long n);
-int launch_chunk_bra(int n_bra, const long long* off, long long n, int* out, cudaStream_t s);
+// bra lookup tables of every class launch
+struct ChunkTable {
+    int n_bra;
+    const long long* off;
+    long long n, entries;
+    int* out;
+};
+struct ChunkTables {
+    ChunkTable t[2 * kNumClasses];
+    int n;
+};
+int launch_chunk_bra(const ChunkTables& c, cudaStream_t s);
 int launch_sum_copies(int n_copies, long long nn, const double* in, double* out, int num_sms, cudaStream_t s);
 int launch_axpby(long long n, const double* A, double alpha, const double* B, double* C, cudaStream_t s);
 int launch_shell_block_max(int n_sh, int N, const int* l, const int* bf0, const double* P, float* dsh, cudaStream_t s);
