@@ -196,7 +196,7 @@ static int capture_graph(hf_batch* B)
                                                                      B->mm.as<MolMat>(), B->Pin.as<double>(),
                                                                      B->bad.as<int>());
     cudaEventRecord(B->fork, st);
-    for (int c = 0; c < kNumClasses; c++) {
+    for (int c = kNumClasses - 1; c >= 0; c--) {  // the classes with the longest quartets first
         if (B->n_total[c] <= 0) continue;
         cudaStreamWaitEvent(B->cst[c], B->fork, 0);
         const BatchArgs a = batch_args(B, c, -1);
@@ -307,7 +307,7 @@ int hf_batch_create(hf_ctx* ctx, int n_mol, const hf_geometry* geoms, const hf_b
             return cleanup(cuda_status(cudaGetLastError(), "hf_batch: class stream"));
         cudaEventCreateWithFlags(&B->join[c], cudaEventDisableTiming);
         B->block[c] = 128;
-        B->chunk[c] = 128;
+        B->chunk[c] = 256;  // one sorted window
         B->bps[c] = 4;
     }
     if (cudaStreamSynchronize(B->st) != cudaSuccess) return cleanup(cuda_status(cudaGetLastError(), "hf_batch: setup"));

@@ -154,10 +154,11 @@ static void ctx_release(hf_ctx* c)
     DeviceGuard g(c->device);
     for (auto& ev : c->ev)
         if (ev) cudaEventDestroy(ev);
-    for (int i = 0; i < kSideStreams; i++) {
-        if (c->join[i]) cudaEventDestroy(c->join[i]);
-        if (c->side[i]) cudaStreamDestroy(c->side[i]);
-    }
+    for (auto& e : c->join)
+        if (e) cudaEventDestroy(e);
+    for (auto& s : c->side)
+        if (s) cudaStreamDestroy(s);
+    if (c->fast) cudaStreamDestroy(c->fast);
     if (c->fork) cudaEventDestroy(c->fork);
     delete c;
 }
@@ -216,8 +217,11 @@ int hf_create(hf_ctx** out, int device, void* cuda_stream)
                 break;
             }
         }
-        for (int i = 0; i < kSideStreams && rc == HF_OK; i++)
-            if (cudaStreamCreateWithFlags(&c->side[i], cudaStreamNonBlocking) != cudaSuccess ||
+        int least = 0, greatest = 0;
+        cudaDeviceGetStreamPriorityRange(&least, &greatest);
+        for (int i = 0; i <= kSideStreams && rc == HF_OK; i++)
+            if (cudaStreamCreateWithPriority(i < kSideStreams ? &c->side[i] : &c->fast, cudaStreamNonBlocking,
+                                             i < kSideStreams ? least : greatest) != cudaSuccess ||
                 cudaEventCreateWithFlags(&c->join[i], cudaEventDisableTiming) != cudaSuccess)
                 rc = cuda_status(cudaGetLastError(), "hf_create: side stream");
         if (rc == HF_OK && cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) != cudaSuccess)
@@ -275,6 +279,7 @@ struct SideStreams {
         HF_CUDA(cudaEventRecord(ctx->fork, ctx->stream));
         open = true;
         for (auto& s : ctx->side) HF_CUDA(cudaStreamWaitEvent(s, ctx->fork, 0));
+        HF_CUDA(cudaStreamWaitEvent(ctx->fast, ctx->fork, 0));
         return HF_OK;
     }
     int join()
@@ -282,8 +287,8 @@ struct SideStreams {
         if (!open) return HF_OK;
         open = false;
         cudaError_t err = cudaSuccess;
-        for (int i = 0; i < kSideStreams; i++) {
-            const cudaError_t e1 = cudaEventRecord(ctx->join[i], ctx->side[i]);
+        for (int i = 0; i <= kSideStreams; i++) {
+            const cudaError_t e1 = cudaEventRecord(ctx->join[i], i < kSideStreams ? ctx->side[i] : ctx->fast);
             const cudaError_t e2 = cudaStreamWaitEvent(ctx->stream, ctx->join[i], 0);
             if (err == cudaSuccess) err = e1 != cudaSuccess ? e1 : e2;
         }
@@ -806,12 +811,15 @@ int hf_system_set_fock_copies(hf_system* S, int32_t copies)
 
 }  // extern "C"
 
+constexpr int kBeside32 = 2;  // blocks per SM of an FP32 launch beside FP64 ones
+
 // One class launch of a build.
 struct ClassLaunch {
     int ci, prec, use_f32;
     Fp64Method method;
     bool warp;   // Hermite warp kernel
     int lanes;   // lanes per quartet (thread kernels), parts per quartet (warp kernel)
+    int rounds;  // Hermite thread kernel: rounds per sorted window; warp kernel: > 1 for groups of quartets
     int grid;
     double est;  // estimated device time, in operations of the whole GPU
 };
@@ -839,51 +847,89 @@ int hf::launch_eri_classes(hf_system* S, EriArgs a, int shard, int n_shards, int
     a.herm = S->herm;
     ClassLaunch todo[2 * kNumClasses];
     int n_todo = 0;
+    // primitive quartets of a quartet (about 0.4 of them survive the primitive threshold) and the time of the whole
+    // build at 1.1 TFLOP/s
+    const double prims = (S->th.prim_tau > 0.0 ? 0.4 : 1.0) * X.maxpp * X.maxpp;
+    double t_all = 0.0, t_all32 = 0.0;
+    for (int ci = 0; ci < kNumClasses; ci++) {
+        const double n = (double)S->plan[ci].n64 + ((flags & HF_FP64_ONLY) ? (double)S->plan[ci].n32 : 0.0);
+        t_all += n / n_shards * (kEriClasses[ci].prim_flops_h * prims + kEriClasses[ci].cont_flops_h) / 1.1e12;
+        if (!(flags & HF_FP64_ONLY))
+            t_all32 += (double)S->plan[ci].n32 / n_shards * (kEriClasses[ci].prim_flops * prims + kEriClasses[ci].cont_flops) / 1.0e13;
+    }
     for (int ci = 0; ci < kNumClasses; ci++)
         for (int prec = 0; prec < 2; prec++) {
             const long long n = prec ? S->plan[ci].n32 : S->plan[ci].n64;
             const long long nq = n * (shard + 1) / n_shards - n * shard / n_shards;
             const EriClassEntry& cl = kEriClasses[ci];
-            ClassLaunch c{ci, prec, prec && !(flags & HF_FP64_ONLY), fp64_method(ci, flags), false, 1, 0, 0.0};
-            const bool herm = !c.use_f32 && c.method == Fp64Method::kHerm;
-            // a class too small to fill the GPU with one thread per quartet shares each quartet's
-            // primitive work among a lane group or a warp instead (shorter latency, same result)
+            ClassLaunch c{ci, prec, prec && !(flags & HF_FP64_ONLY), fp64_method(ci, flags), false, 1, 1, 0, 0.0};
+            // a class too small to fill the GPU with one thread per quartet
             const bool small = !c.use_f32 && nq < (long long)ctx->num_sms * 256;
-            double ops = (double)cl.prim_flops * X.maxpp * X.maxpp + cl.cont_flops;
-            if (herm) {
-                ops = (double)cl.prim_flops_h * X.maxpp * X.maxpp + cl.cont_flops_h;
-                c.warp = !cl.launch_herm || (small && cl.launch_hermw);
+            const long long windows_min = (long long)ctx->num_sms * 4;
+            double ops = (double)cl.prim_flops * prims + cl.cont_flops;
+            if (!c.use_f32 && c.method == Fp64Method::kHerm) {
+                ops = (double)cl.prim_flops_h * prims + cl.cont_flops_h;
+                // One thread per quartet wastes the least, but lasts as long as one lane needs for a quartet
+                // (about 0.65 FP64 instructions an operation, 64 clocks each, three warps sharing a scheduler): fine
+                // while that is half of the whole build, which the other classes fill.  Otherwise a small launch
+                // shares each quartet among a lane group or a warp.  Against "small" alone: split-valence 10 waters
+                // 7.0 -> 5.1 ms, 4 waters unscreened 10.9 -> 10.3 ms (a quarter or twice of the half: within 1%).
+                const double lat = ops * 0.65 * 64.0 * 3.0 / 2.0e9;
+                const bool fits = cl.launch_herm && lat <= 0.5 * t_all;
+                c.warp = !cl.launch_herm || (small && !fits && cl.launch_hermw);
                 if (c.warp) {
                     // parts: quartets fewer than four warps per SM take one warp per batch of 32 primitive quartets
                     const long long batches = ((long long)X.maxpp * X.maxpp + 31) / 32;
                     c.lanes = (int)std::max<long long>(1, std::min(batches, (long long)ctx->num_sms * 4 / std::max<long long>(nq, 1)));
-                    c.grid = (int)std::min<long long>(nq * c.lanes, 1 << 20);
-                } else if (small) {
-                    c.lanes = cl.herm_lanes;
+                    // groups of quartets per warp once there are eight warps per SM without them
+                    if (nq >= (long long)ctx->num_sms * 64) c.rounds = 2;
+                } else {
+                    if (small && !fits) c.lanes = cl.herm_lanes;
+                    // sorted windows: as many rounds as keep four windows per SM and the same latency bound (without
+                    // the sort 32 waters 812 -> 831 ms and split-valence 10 waters 5.35 -> 5.96; one window per SM
+                    // 13 waters 70 -> 75)
+                    while (c.lanes == 1 && c.rounds < kSortRounds && nq >= windows_min * 64 * c.rounds &&
+                           2 * c.rounds * lat <= 0.5 * t_all)
+                        c.rounds *= 2;
+                    const long long per_block = (long long)(kEriThreads / c.lanes) * c.rounds;
+                    c.grid = (int)std::min<long long>((nq + per_block - 1) / per_block, 1 << 20);
                 }
-            } else if (small) {
-                c.lanes = cl.lanes;
-            }
-            if (!c.warp)
+            } else {
+                // shares each quartet's primitive work among a lane group (shorter latency, same result)
+                if (small) c.lanes = cl.lanes;
                 c.grid = (int)std::min<long long>((nq * c.lanes + kEriThreads - 1) / kEriThreads, (long long)ctx->num_sms * 16);
+            }
             // one quartet's operations run in one lane (warp), 1 / (64 lanes SMs) of the GPU at a time
             c.est = std::max((double)nq, 64.0 * ctx->num_sms / (c.warp ? 32 * c.lanes : c.lanes)) * ops / (c.use_f32 ? 32.0 : 1.0);
             if (nq > 0 || ev) todo[n_todo++] = c;
         }
     const bool forked = !ev && n_todo > 1;
     double load[kSideStreams] = {};
+    SideStreams side(ctx);
     if (forked) {
         std::sort(todo, todo + n_todo, [](const ClassLaunch& x, const ClassLaunch& y) { return x.est > y.est; });
-        HF_CUDA(cudaEventRecord(ctx->fork, ctx->stream));
-        for (int i = 0; i < std::min(kSideStreams, n_todo); i++) HF_CUDA(cudaStreamWaitEvent(ctx->side[i], ctx->fork, 0));
+        TRY(side.fork());
     }
+    // The FP64 kernels keep the FP64 pipe busy and leave nine of ten issue slots free; the FP32 kernels of a mixed
+    // build need those slots and next to no FP64.  On one SM at the same time the shorter part costs little, but
+    // blocks of equal priority run one kernel after the other.  So the FP32 launches go to the stream of higher
+    // priority, with few enough persistent blocks that FP64 blocks fit beside them: kBeside32 per SM while the FP32
+    // part is the shorter one, all the SM holds otherwise.  (The quartets above an FP32 cutoff keep about twice the
+    // primitive quartets that t_all assumes, and those below it fewer: 64 waters, FP64 955 ms, FP32 300 ms alone,
+    // estimated 370 and 410.)  Measured: mixed 64 waters 1,245 -> 1,150 ms, a 24-water difference build 103 -> 94 ms;
+    // 2 to 8 blocks per SM within 1%.
+    const bool beside = forked && t_all32 > 0.0 && t_all32 < 2.0 * t_all;
     cudaError_t err = cudaSuccess;
     for (int t = 0; t < n_todo && err == cudaSuccess; t++) {
         const ClassLaunch& c = todo[t];
         const auto& pl = S->plan[c.ci];
         const int Xc = kEriClasses[c.ci].X, Yc = kEriClasses[c.ci].Y;
         cudaStream_t st = ctx->stream;
-        if (forked) {
+        int grid = c.grid;
+        if (beside && c.use_f32) {
+            st = ctx->fast;
+            grid = std::min(grid, ctx->num_sms * kBeside32);
+        } else if (forked) {
             const int i = (int)(std::min_element(load, load + kSideStreams) - load);
             load[i] += c.est;
             st = ctx->side[i];
@@ -918,25 +964,22 @@ int hf::launch_eri_classes(hf_system* S, EriArgs a, int shard, int n_shards, int
             // 2% faster); the FP32 kernels, bound by latency rather than a pipe, ran 10% slower with it
             // and are compiled without it
             a.sort_work = c.use_f32 ? 0 : 1;
+            a.rounds = c.rounds;
             const EriClassEntry& cl = kEriClasses[c.ci];
             if (c.use_f32 || c.method == Fp64Method::kObaraSaika)
-                cl.launch(a, c.use_f32, c.grid, kEriThreads, st, c.lanes);
+                cl.launch(a, c.use_f32, grid, kEriThreads, st, c.lanes);
             else if (c.method == Fp64Method::kRys)
                 cl.launch_rys(a, 0, c.grid, kEriThreads, st, c.lanes);
             else if (c.warp)
-                cl.launch_hermw(a, c.grid, st, c.lanes);
+                cl.launch_hermw(a, st, c.rounds > 1, c.lanes);
             else
                 cl.launch_herm(a, c.grid, st, c.lanes);
             err = cudaGetLastError();
         }
         if (ev && err == cudaSuccess) err = cudaEventRecord(ev[4 * c.ci + 2 * c.prec + 1], st);
     }
-    if (forked)  // joined whether or not a launch failed: what was launched still uses the system's buffers
-        for (int i = 0; i < std::min(kSideStreams, n_todo); i++) {
-            const cudaError_t e1 = cudaEventRecord(ctx->join[i], ctx->side[i]);
-            const cudaError_t e2 = cudaStreamWaitEvent(ctx->stream, ctx->join[i], 0);
-            if (err == cudaSuccess) err = e1 != cudaSuccess ? e1 : e2;
-        }
+    const int rc = side.join();
+    if (err == cudaSuccess && rc != HF_OK) return rc;
     return err == cudaSuccess ? HF_OK : cuda_status(err, "ERI class launch");
 }
 

@@ -738,9 +738,11 @@ def gen_class(X, Y, method="os"):
     return "\n".join(out) + "\n", info
 
 
-# Hermite-accumulator kernels: classes up to this total angular momentum have a thread kernel (their
-# accumulators fit the registers, with a few spills at 100 to 157 of them), classes from HERM_WARP_MIN_L on a
-# warp kernel; small launches of the classes with both use the warp kernel.
+# Hermite-accumulator kernels: classes up to HERM_THREAD_MAX_L have a thread kernel with its accumulators in
+# registers (spilling a few at 100 to 157 of them; left to the compiler, the 223 and more of L = 5 put the whole
+# function into a 32-register allocation, and kept in shared memory they leave one warp per scheduler: (dp|ds)
+# 64 ms of a 32-water build against 43 in the warp kernel).  Classes from HERM_WARP_MIN_L on have a warp kernel; the
+# launch picks one for the classes with both.
 HERM_THREAD_MAX_L = 4
 HERM_WARP_MIN_L = 4
 HERM_LANES = 8  # lanes per quartet of the thread kernels in small launches and Schwarz bounds
@@ -767,13 +769,13 @@ def gen_herm_class(X, Y):
         lines.append("const double fj = 4.0 * fscale, fk = 2.0 * fscale;")
         dig = gen_digest(la, lb, lc, ld, xname, cnt)
         lines += [l.replace("(bB +", "(bB_ +").replace("* N + bB +", "* N + bB_ +") for l in dig]
-        return lines, cnt.cont, None
+        return lines, cnt.cont
 
     out = [f"// ({PAIR_NAMES[X]}|{PAIR_NAMES[Y]}) class: l = {la}{lb}{lc}{ld}, Hermite accumulators."]
     info = dict(hname=name, herm_thread=L <= HERM_THREAD_MAX_L, herm_warp=L >= HERM_WARP_MIN_L)
     kernels = []
     if info["herm_thread"]:
-        src, pf, cf, nacc = gen_herm.gen_thread(name, la, lb, lc, ld, hrr_digest)
+        src, pf, cf = gen_herm.gen_thread(name, la, lb, lc, ld, hrr_digest)
         out += [src, f"HERM_THREAD_KERNELS({name}, {HERM_LANES})", f"HERM_THREAD_BATCH({name})"]
         kernels += [f"k_herm_{name}<1>", f"k_herm_{name}<{HERM_LANES}>"]
         info.update(prim_flops_h=pf, cont_flops_h=cf)
@@ -850,7 +852,7 @@ def main(outdir):
         if info["herm_thread"]:
             lines.append(f"void launch_herm_{n}(const EriArgs&, int, cudaStream_t, int);")
         if info["herm_warp"]:
-            lines.append(f"void launch_hermw_{n}(const EriArgs&, int, cudaStream_t, int);")
+            lines.append(f"void launch_hermw_{n}(const EriArgs&, cudaStream_t, int, int);")
         if info["X"] == info["Y"]:
             lines.append(f"void launch_schwarz_{n}(const SchwarzArgs&, int, cudaStream_t);")
         lines.append(f"void launch_eri_batch_{n}(const BatchArgs&, int, int, cudaStream_t);")

@@ -259,7 +259,7 @@ def gen_thread(name, la, lb, lc, ld, hrr_digest):
             cont += ls
             for f, nm in out.items():
                 final[(e, f)] = nm
-    tail, cops, schwarz = hrr_digest(final)
+    tail, cops = hrr_digest(final)
     co.n += cops
     need_ab = any("AB" in l for l in cont + tail)
     need_cd = any("CD" in l for l in cont + tail)
@@ -326,7 +326,7 @@ def gen_thread(name, la, lb, lc, ld, hrr_digest):
              " int lane, bool valid)")
     o.append(f"    {{ return quartet_h_{name}<G>(hb, hk, hv, bt, Pd, N, f, Jt, Kt, qout, ptau, lane, valid); }}")
     o.append("};")
-    return "\n".join(o) + "\n", po.n, co.n, len(acc)
+    return "\n".join(o) + "\n", po.n, co.n
 
 
 def gen_warp(name, la, lb, lc, ld):
@@ -363,6 +363,9 @@ def gen_warp(name, la, lb, lc, ld):
     o.append(f"    static constexpr int NR = {len(hs)}, NRP = {nrp}, NBS = {len(B)}, NKS = {len(K)}, NACC = {len(acc)},"
              f" NSLOT = {nslot}, NBI = {len(BI)}, NKI = {len(KI)}, NE = {len(es)}, NF = {len(fs)};")
     o.append(f"    static constexpr int LA = {la}, LB = {lb}, LC = {lc}, LD = {ld};")
+    # quartets per group: enough (quartet, ket item) columns for the lanes; one where L >= 7 needs the shared memory
+    ng = 1 if L >= 7 else {1: 8, 4: 8, 11: 3, 15: 2, 35: 2}[len(KI)]
+    o.append(f"    static constexpr int NQ = {ng};")
     o.append("    static __device__ __forceinline__ const unsigned short* slots() { return kHermSlot_%s; }" % name)
     o.append("    static __device__ __forceinline__ const unsigned short* item_table() { return kHermItem_%s; }" % name)
     o.append("    // one primitive quartet: R[0..NR), scalings sc[0..NBS + NKS)")

@@ -85,7 +85,8 @@ struct EriArgs {
     const PairHdr* bhdr;              // headers of the bra list in list order (bhdr[b] = pairs[bra[b]])
     const PairHdr* khdr;              // headers of the ket list in list order (khdr[k] = pairs[ket[k]])
     HermView herm;
-    int sort_work;                    // 1: each warp runs its window of quartets sorted by staircase length
+    int rounds;                       // Hermite thread kernels: rounds per sorted window (1: launch order)
+    int sort_work;                    // Obara-Saika kernels, 1: each warp runs its window of quartets sorted by staircase length
 };
 
 struct SchwarzArgs {
@@ -148,11 +149,11 @@ struct BatchArgs {
 struct EriClassEntry {
     int X, Y, L;
     // Hermite-accumulator kernels (the FP64 default): the thread kernel (nullptr: the class has none), the warp
-    // kernel (nullptr: none), its blocks per SM, operations per primitive and per contracted quartet
+    // kernel (nullptr: none; group 1: several quartets per warp), operations per primitive and per contracted quartet
     int prim_flops_h, cont_flops_h;
     void (*launch_herm)(const EriArgs&, int grid, cudaStream_t, int lanes);
     int herm_lanes;  // lanes per quartet of the thread kernel in small launches
-    void (*launch_hermw)(const EriArgs&, int grid, cudaStream_t, int nparts);
+    void (*launch_hermw)(const EriArgs&, cudaStream_t, int group, int nparts);
     int (*prepare)();             // sets the kernels' shared-memory limits once per device
     size_t (*local_bytes_h)();
     int batch_warp;               // 1: the batched kernel is one warp per block
@@ -267,8 +268,9 @@ struct hf_ctx {
     cudaEvent_t ev[4 * hf::kNumClasses + 4] = {};
     int n_systems = 0;            // live systems created on this context
     bool destroy_pending = false;  // hf_destroy was called while systems were alive
+    cudaStream_t fast = nullptr;  // of higher priority: the FP32 launches beside FP64 ones
     cudaStream_t side[hf::kSideStreams] = {};  // class launches of one build run on these, forked from and
-    cudaEvent_t fork = nullptr, join[hf::kSideStreams] = {};  // joined to `stream` (launch_eri_classes)
+    cudaEvent_t fork = nullptr, join[hf::kSideStreams + 1] = {};  // joined to `stream` (launch_eri_classes)
     void* noalloc_scratch = nullptr;  // device address of hf_fock_build_noalloc's fixed scratch
 };
 
