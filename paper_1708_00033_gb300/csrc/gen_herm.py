@@ -82,10 +82,13 @@ class Ops:
         self.n = 0
 
 
-def scale_lines(la, lb, rec, pre, ops):
-    """Lines computing u^k v^(W-k-s) of every scaling; returns (lines, [name or None for 1])."""
+def scale_lines(la, lb, rec, pre, ops, start=None):
+    """Lines computing start u^k v^(W-k-s) of every scaling, each from another by one multiplication (start: a
+    factor, or None for 1); returns (lines, [name or None for 1])."""
     W = la + lb
-    have = {(0, 0): None, (1, 0): f"{rec}.u", (0, 1): f"{rec}.v"}
+    have = {(0, 0): start}
+    if start is None:
+        have.update({(1, 0): f"{rec}.u", (0, 1): f"{rec}.v"})
     lines = []
 
     def need(k, m):
@@ -102,9 +105,11 @@ def scale_lines(la, lb, rec, pre, ops):
     return lines, [need(k, W - k - s) for (k, s) in scalings(la, lb)]
 
 
-def r_lines(L, ops):
+def r_lines(L, ops, leaf_orders=()):
     """Hermite Coulomb integrals r_N^(0) from g_m = (2 rho)^m F_m and the separation D = Q - P: with
-    q^(m) = (-1)^m R^(m), q_{N+1_i}^(m) = D_i q_N^(m+1) - N_i q_{N-1_i}^(m+1)."""
+    q^(m) = (-1)^m R^(m), q_{N+1_i}^(m) = D_i q_N^(m+1) - N_i q_{N-1_i}^(m+1).  Returns (lines, name of r_N,
+    terms), terms(N) = [(axis or None, factor, name)]: r_N as a sum of D_axis * name and -factor * name.  No other
+    r depends on an r_N^(0), so those of leaf_orders are not formed: the caller accumulates their terms."""
     recipe = {}
 
     def need(t, m):
@@ -127,6 +132,8 @@ def r_lines(L, ops):
     for (t, m), i in sorted(recipe.items(), key=lambda kv: (sum(kv[0][0]), -kv[0][1])):
         if i is None:
             continue
+        if m == 0 and sum(t) in leaf_orders:
+            continue
         e = f"D{AX[i]} * {nm(add(t, i, -1), m + 1)}"
         ops.n += 1
         if t[i] >= 2:
@@ -134,11 +141,20 @@ def r_lines(L, ops):
             e += (" - " if c == 1 else f" - {c}.0 * ") + nm(add(t, i, -2), m + 1)
             ops.n += 1 if c == 1 else 2
         lines.append(f"const double {nm(t, m)} = {e};")
-    return lines, lambda t: nm(t, 0)
+
+    def terms(t):
+        i = recipe[(t, 0)]
+        out = [(i, 1, nm(add(t, i, -1), 1))]
+        if t[i] >= 2:
+            out.append((None, t[i] - 1, nm(add(t, i, -2), 1)))
+        return out
+
+    return lines, (lambda t: nm(t, 0)), terms
 
 
-def prim_lines(la, lb, lc, ld, ops):
-    """One primitive quartet up to g_m, the scalings and r_N: (lines, r name, bra names, ket names)."""
+def prim_lines(la, lb, lc, ld, ops, leaf_orders=()):
+    """One primitive quartet up to g_m, the scalings and r_N: (lines, r name, r terms, bra names, ket names).  The
+    prefactor is part of the bra scalings."""
     L = la + lb + lc + ld
     lines = ["const double Dx = kp.Px - bp.Px, Dy = kp.Py - bp.Py, Dz = kp.Pz - bp.Pz;",
              "double rs, a2;",
@@ -156,20 +172,10 @@ def prim_lines(la, lb, lc, ld, ops):
             lines.append(f"const double a2_{m + 1} = {pw} * a2;")
             ops.n += 1
             pw = f"a2_{m + 1}"
-    b, bn = scale_lines(la, lb, "bp", "ub", ops)
+    b, bn = scale_lines(la, lb, "bp", "sb", ops, "pf")
     k, kn = scale_lines(lc, ld, "kp", "uk", ops)
-    r, rname = r_lines(L, ops)
-    # the prefactor goes into the bra scalings
-    lines += b + k
-    names = []
-    for i, n in enumerate(bn):
-        if n is None:
-            names.append("pf")
-        else:
-            lines.append(f"const double sb{i} = pf * {n};")
-            ops.n += 1
-            names.append(f"sb{i}")
-    return lines + r, rname, names, kn
+    r, rname, terms = r_lines(L, ops, leaf_orders)
+    return lines + b + k + r, rname, terms, bn, kn
 
 
 def transform(la, lb, src, ab, ket, ops, pre):
@@ -226,7 +232,14 @@ def gen_thread(name, la, lb, lc, ld, hrr_digest):
     L = la + lb + lc + ld
     acc = accumulators(la, lb, lc, ld)
     po, co = Ops(), Ops()
-    lines, rname, bn, kn = prim_lines(la, lb, lc, ld, po)
+    # r_N that few scalings use are accumulated from their terms with the scaling folded into D (p D_i once per
+    # scaling): the top order, which one scaling uses, and order 1 when fewer than three do
+    uses = {}
+    for (i, j) in {(i, j) for i, j, _ in acc}:
+        for n in {sum(t) for a, b, t in acc if (a, b) == (i, j)}:
+            uses[n] = uses.get(n, 0) + 1
+    leaf = {n for n in uses if n >= 1 and ((n == L and L != 2) or (n == 1 and uses[n] < 3))}
+    lines, rname, terms, bn, kn = prim_lines(la, lb, lc, ld, po, leaf)
     body = list(lines)
     order = {}
     for idx, (i, j, t) in enumerate(acc):
@@ -238,9 +251,33 @@ def gen_thread(name, la, lb, lc, ld, hrr_digest):
             p = f"s{i}_{j}"
             body.append(f"const double {p} = {bn[i]} * {kn[j]};")
             po.n += 1
+        made = set()
+
+        def coef(name, expr):
+            if name not in made:
+                made.add(name)
+                body.append(f"const double {name} = {expr};")
+                po.n += 1
+            return name
+
         for idx, t in ts:
-            body.append(f"h{idx} = fma({p}, {rname(t)}, h{idx});")
-            po.n += 2
+            if sum(t) not in leaf:
+                body.append(f"h{idx} = fma({p}, {rname(t)}, h{idx});")
+                po.n += 2
+            elif sum(t) == 1:  # D_i (p g_1)
+                ax, _, nm = terms(t)[0]
+                body.append(f"h{idx} = fma(D{AX[ax]}, {coef(f'pg{i}_{j}', f'{p} * {nm}')}, h{idx});")
+                po.n += 2
+            else:
+                for ax, c, nm in terms(t):
+                    if ax is not None:
+                        k = coef(f"pD{AX[ax]}{i}_{j}", f"{p} * D{AX[ax]}")
+                    elif c == 1:
+                        k = f"-{p}"
+                    else:
+                        k = coef(f"pn{c}_{i}_{j}", f"-{c}.0 * {p}")
+                    body.append(f"h{idx} = fma({k}, {nm}, h{idx});")
+                    po.n += 2
     B, K = list(scalings(la, lb)), list(scalings(lc, ld))
     where = {(B[i], K[j], t): f"h{idx}" for idx, (i, j, t) in enumerate(acc)}
     cont = []
@@ -339,7 +376,7 @@ def gen_warp(name, la, lb, lc, ld):
     BI, KI = items(la, lb), items(lc, ld)
     where = {(B[i], K[j], t): a for a, (i, j, t) in enumerate(acc)}
     po, co = Ops(), Ops()
-    lines, rname, bn, kn = prim_lines(la, lb, lc, ld, po)
+    lines, rname, _, bn, kn = prim_lines(la, lb, lc, ld, po)
     po.n += sum(1 for n in kn if n is not None) * len(bn) + 2 * len(acc)
     es = [e for n in range(la, la + lb + 1) for e in CART[n]]
     fs = [f for n in range(lc, lc + ld + 1) for f in CART[n]]
@@ -443,17 +480,15 @@ def gen_onee(la, lb):
         if m:
             o.append("        zp *= bp.v;")
         o.append(f"        const double g{m} = zp * F[{m}];")
-    lines, rname = r_lines(L, ops)
+    lines, rname, _ = r_lines(L, ops)
     o += ["        " + l for l in lines]
     o += [f"        RS[{i}] += {rname(t)};" for i, t in enumerate(hs)]
     o += ["    }", "    // acc += pf sigma RS_N of every scaling and order",
           "    static __device__ __forceinline__ void scale(const HermPair& bp, double pf, const double (&RS)[NR], double (&acc)[NI])",
           "    {"]
-    lines, names = scale_lines(la, lb, "bp", "ub", ops)
+    lines, names = scale_lines(la, lb, "bp", "sb", ops, "pf")
     o += ["        " + l for l in lines]
-    for i, n in enumerate(names):
-        o.append(f"        const double sb{i} = pf" + (f" * {n};" if n else ";"))
-    o += [f"        acc[{x}] = fma(sb{sc.index((k, s))}, RS[{hidx[t]}], acc[{x}]);" for x, (k, s, t) in enumerate(its)]
+    o += [f"        acc[{x}] = fma({names[sc.index((k, s))]}, RS[{hidx[t]}], acc[{x}]);" for x, (k, s, t) in enumerate(its)]
     o += ["    }", "    // (a|b) from the accumulators",
           "    static __device__ __forceinline__ void finish(const double (&acc)[NI], double ABx, double ABy, double ABz, double* __restrict__ V)",
           "    {"]
