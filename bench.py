@@ -36,12 +36,10 @@ DFMA_PEAK_GFLOPS = 152 * 2 * 2 * 2.070  # 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of the dominant kernel, from one
 # ncu capture of the default workload, with the SHA-256 of the sources that kernel is compiled from at that
 # time; the bench reports it only while those sources are unchanged (else the counters describe another
-# kernel and traffic is null).  Capture: the 64-water FP64 build at the bench's thresholds (`--mode case
-# --case fock --waters 64`), one pass, both launches of k_eri_1110<double>: 3.79 GB + 630.90 MB and
-# 3.80 GB + 632.54 MB; their mean.
-NCU_TRAFFIC = {"kernel": "k_eri_1110", "bytes_per_launch": 4.4267e9,
-               "sources_sha256": "18cdc26cad87ad9d767e774a67808fd25df6ef1a68ef13699d23cc8cda1164c0"}
-TRAFFIC_SOURCES = ("paper_1708_00033_gb300/csrc/gen_eri.py", "paper_1708_00033_gb300/csrc/eri_common.cuh",
+# kernel and traffic is null).
+NCU_TRAFFIC = {"kernel": "k_herm_1110", "bytes_per_launch": None, "sources_sha256": None}
+TRAFFIC_SOURCES = ("paper_1708_00033_gb300/csrc/gen_eri.py", "paper_1708_00033_gb300/csrc/gen_herm.py",
+                   "paper_1708_00033_gb300/csrc/eri_common.cuh", "paper_1708_00033_gb300/csrc/eri_herm.cuh",
                    "paper_1708_00033_gb300/csrc/hf_internal.h")
 
 
@@ -59,6 +57,15 @@ def measured_traffic(kernel: str):
     if NCU_TRAFFIC["kernel"] != kernel or NCU_TRAFFIC["bytes_per_launch"] is None:
         return None
     return NCU_TRAFFIC["bytes_per_launch"] if kernel_sources_sha256() == NCU_TRAFFIC["sources_sha256"] else None
+
+
+def fp64_kernel(hf, c: int) -> str:
+    """Name of the FP64 kernel that large launches of class c run by default (one thread per quartet up to a total
+    angular momentum of 4, one warp above)."""
+    name = hf.CLASS_KERNELS[c][-4:]
+    return ("k_herm_" if sum(map(int, name)) <= 4 else "k_hermw_") + name
+
+
 L2_BYTES = 129 * 2 ** 20
 
 
@@ -222,13 +229,15 @@ def run_ours(a):
         flush.zero_()  # L2 flush between timed steps (outside the events)
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         e0.record(stream)
-        out = sysm.fock_build(Pd, F=Fd, timing=True)
+        out = sysm.fock_build(Pd, F=Fd, stats=True)
         e1.record(stream)
         torch.cuda.synchronize()
         step_ms.append(e0.elapsed_time(e1))
         stats.append(out["stats"])
     torch.cuda.synchronize()
     clk = clocks.stop()
+    # device time per class: one more build, whose class launches run one after another instead of concurrently
+    timed = sysm.fock_build(Pd, F=Fd, timing=True)["stats"]
     total_ms = sum(step_ms)
     if world > 1:
         total_ms = reduce_max(total_ms, dist, dev)
@@ -253,11 +262,11 @@ def run_ours(a):
                "d2h_bytes_per_step": N * N * 8 + 8}
 
     # roofline of the dominant kernel (the class kernel with the largest device time)
-    ms_cls = np.mean([s["ms_class_fp64"] for s in stats], axis=0) + np.mean([s["ms_class_fp32"] for s in stats], axis=0)
+    ms_cls = np.array(timed["ms_class_fp64"]) + np.array(timed["ms_class_fp32"])
     c = int(np.argmax(ms_cls))
     fl = stats[0]["class_flops_fp64"][c] + stats[0]["class_flops_fp32"][c]
     achieved = fl / (ms_cls[c] / 1e3) / 1e9
-    eri_ms = float(np.mean([s["ms_eri"] for s in stats]))
+    eri_ms = float(timed["ms_eri"])
     eri_gflops = (stats[0]["flops_fp64"] + stats[0]["flops_fp32"]) / (eri_ms / 1e3) / 1e9
     line = {
         "metric": "Fock builds/s",
@@ -282,9 +291,9 @@ def run_ours(a):
                    "l2": "flushed between timed steps (256 MiB write)", "parallelism": f"replicas x{world}"},
         "gpu_launches": int(sum(s["kernels_launched"] for s in stats)),
         "clocks": clk,
-        "roofline": {"bound": "alu", "kernel": hf.CLASS_KERNELS[c], "class": hf.CLASS_NAMES[c], "achieved": achieved,
+        "roofline": {"bound": "alu", "kernel": fp64_kernel(hf, c), "class": hf.CLASS_NAMES[c], "achieved": achieved,
                      "peak": DFMA_PEAK_GFLOPS, "unit": "GFLOP/s", "frac": achieved / DFMA_PEAK_GFLOPS,
-                     "traffic": measured_traffic(hf.CLASS_KERNELS[c]),
+                     "traffic": measured_traffic(fp64_kernel(hf, c)),
                      "peak_kind": "FP64 FMA pipe, derived from unit counts and max clock (hf_measure_peaks: 1,252)",
                      "all_eri_kernels": {"ms": eri_ms, "achieved": eri_gflops,
                                          "frac": eri_gflops / DFMA_PEAK_GFLOPS}},

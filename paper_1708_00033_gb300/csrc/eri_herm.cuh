@@ -208,7 +208,7 @@ __device__ __forceinline__ double herm_norm2(int l, int c) { return l == 2 && (c
 // room for warps run several parts per quartet.
 template <class C, class Fetch>
 __device__ __forceinline__ int herm_warp(int g, Fetch fetch, const double2* __restrict__ etab, int ntype,
-                                         const double* __restrict__ boys_tab, double* qout, int part, int nparts,
+                                         const double* __restrict__ boys_tab, bool schwarz, int part, int nparts,
                                          double* __restrict__ sh)
 {
     using Z = HermShape<C>;
@@ -341,13 +341,17 @@ __device__ __forceinline__ int herm_warp(int g, Fetch fetch, const double2* __re
     }
     __syncwarp();
     if constexpr (C::LA == C::LC && C::LB == C::LD) {
-        if (qout) {  // Schwarz bound: max |(ab|ab)| of normalised components
-            double m = 0.0;
-            for (int ab = lane; ab < Z::NAB; ab += 32)
-                m = fmax(m, fabs(H[ab * Z::NCD + ab]) * herm_norm2(C::LA, ab / Z::NB) * herm_norm2(C::LB, ab % Z::NB));
+        if (schwarz) {  // Schwarz bound sqrt(max |(ab|ab)|) of normalised components, to the descriptor's J
+            for (int q = 0; q < g; q++) {
+                if (Q[q].nb == 0) continue;
+                double m = 0.0;
+                for (int ab = lane; ab < Z::NAB; ab += 32)
+                    m = fmax(m, fabs(H[q * Z::nH + ab * Z::NCD + ab]) * herm_norm2(C::LA, ab / Z::NB) *
+                                    herm_norm2(C::LB, ab % Z::NB));
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(full, m, o));
-            if (lane == 0) *qout = m;
+                for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(full, m, o));
+                if (lane == 0) *Q[q].J = sqrt(m);
+            }
             __syncwarp();
             return nq;
         }
@@ -426,7 +430,7 @@ __device__ __forceinline__ void herm_warp_kernel(const EriArgs& a, int g, int np
             d.K = a.Kt + cofs;
             d.N = a.N;
         };
-        nprimq += herm_warp<C>((int)min((long long)g, a.n_quartets - q0), fetch, hv.etab, hv.ntype, a.boys64, nullptr,
+        nprimq += herm_warp<C>((int)min((long long)g, a.n_quartets - q0), fetch, hv.etab, hv.ntype, a.boys64, false,
                                (int)(w % nparts), nparts, sh);
     }
     if (a.prim_count) {
@@ -435,7 +439,8 @@ __device__ __forceinline__ void herm_warp_kernel(const EriArgs& a, int g, int np
     }
 }
 
-// item 0 of a pair: its contracted bound; item i > 0: primitive pair i - 1 alone (see SCHWARZ_KERNEL)
+// Schwarz bounds: item 0 of a pair is Q = sqrt(max |(ab|ab)|) of the contracted pair, item i > 0 the same bound of
+// primitive pair i - 1 alone
 struct SchwarzItem {
     PairHdr h;
     double* out;
@@ -456,7 +461,7 @@ struct SchwarzItem {
     }
 };
 
-// Work queue of a batched build (see ERI_BATCH_KERNEL): (molecule, bra, ket) of quartet q.
+// Batched build: (molecule, bra, ket) of quartet q of the batch's index space.
 __device__ __forceinline__ void batch_quartet(const BatchArgs& a, long long q, int& m, int& b, int& k)
 {
     m = find_bra(a.mol_off, a.n_mol, q);
@@ -538,7 +543,7 @@ __device__ __forceinline__ void herm_warp_batch(const BatchArgs& a, double* sh)
             d.K = mc.Kt;
             d.N = mc.N;
         };
-        herm_warp<C>((int)min((long long)C::NQ, a.n_total - (long long)q0), fetch, hv.etab, hv.ntype, a.boys64, nullptr, 0,
+        herm_warp<C>((int)min((long long)C::NQ, a.n_total - (long long)q0), fetch, hv.etab, hv.ntype, a.boys64, false, 0,
                      1, sh);
     }
 }
@@ -592,7 +597,7 @@ inline size_t herm_local_bytes(K... kernels)
         k_hermw_##NAME<<<grid, 32, HermShape<HermWarp_##NAME>::bytes, s>>>(a, g, nparts);                    \
     }
 
-// Schwarz bounds of a diagonal class: 8 lanes (thread form) or one warp per item.
+// Schwarz bounds of a diagonal class: 8 lanes (thread form) per item or one warp per group of items.
 #define HERM_THREAD_SCHWARZ(NAME)                                                                            \
     __global__ void __launch_bounds__(kEriThreads) k_schwarz_##NAME(const SchwarzArgs a)                    \
     {                                                                                                        \
@@ -612,21 +617,21 @@ inline size_t herm_local_bytes(K... kernels)
     __global__ void __launch_bounds__(32) k_schwarz_##NAME(const SchwarzArgs a)                             \
     {                                                                                                        \
         extern __shared__ double hsh[];                                                                      \
-        const SchwarzItem it(a, blockIdx.x);                                                                 \
-        if (!it.valid) return; /* block-uniform */                                                           \
-        double qm = 0.0;                                                                                     \
-        auto fetch = [&](int, HermQuartet& d) {                                                              \
+        constexpr int g = HermWarp_##NAME::NQ; /* items per warp: most are single primitive pairs */         \
+        auto fetch = [&](int i, HermQuartet& d) {                                                            \
+            const SchwarzItem it(a, (long long)blockIdx.x * g + i);                                          \
+            if (!it.valid) return;                                                                           \
             d.set(it.h, it.h, a.herm);                                                                       \
             d.ptau = 0.0f;                                                                                   \
+            d.J = it.out;                                                                                    \
         };                                                                                                   \
-        herm_warp<HermWarp_##NAME>(1, fetch, a.herm.etab, a.herm.ntype, a.boys64, &qm, 0, 1, hsh);           \
-        if (threadIdx.x == 0) *it.out = sqrt(qm);                                                            \
+        herm_warp<HermWarp_##NAME>(g, fetch, a.herm.etab, a.herm.ntype, a.boys64, true, 0, 1, hsh);          \
     }                                                                                                        \
     void launch_schwarz_##NAME(const SchwarzArgs& a, int, cudaStream_t s)                                   \
     {                                                                                                        \
         if (cudaFuncSetAttribute(k_schwarz_##NAME, cudaFuncAttributeMaxDynamicSharedMemorySize,              \
                                  (int)HermShape<HermWarp_##NAME>::bytes) != cudaSuccess) return;             \
-        const long long items = (long long)a.n * a.items;                                                    \
+        const long long items = ((long long)a.n * a.items + HermWarp_##NAME::NQ - 1) / HermWarp_##NAME::NQ;  \
         if (items > 0) k_schwarz_##NAME<<<(unsigned)items, 32, HermShape<HermWarp_##NAME>::bytes, s>>>(a);   \
     }
 

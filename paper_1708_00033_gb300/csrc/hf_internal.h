@@ -46,6 +46,8 @@ struct HermView {
     const double2* etab;
     int ntype;
 };
+constexpr double kPairPrefactor = 5.914967172795613;  // sqrt(2) pi^(5/4): two pairs' product is 2 pi^(5/2)
+constexpr double kNuclearPrefactor = 1.0622519320271968;  // 2 pi / kPairPrefactor (as rounded)
 constexpr int kHermMaxTypes = 1448;  // 32 MB of exponent table
 
 struct EriArgs {

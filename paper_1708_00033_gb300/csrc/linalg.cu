@@ -7,7 +7,6 @@
 //     of V' = V J being independent; one launch per round, ping-pong buffers;
 //   - small helpers (antisymmetric part, dot products, linear combinations,
 //     RMS difference, the Pulay DIIS system solved on the device).
-#include <cooperative_groups.h>
 #include <math.h>
 
 #include <utility>
@@ -364,9 +363,8 @@ __global__ void k_drop_index(int m, int* perm, int x)
 // already diagonal to its own tolerance, or nearly so (clustered eigenvalues), and its convergence test decides
 // as before.
 //   1. One-sided (Hestenes) Jacobi in FP32 on the columns of G = A / s + c I, c > ||A / s||: G is positive
-//      definite, so its columns converge to lambda_j v_j and need no second matrix.  One warp per column pair, one
-//      barrier per round; the whole matrix in one SM's shared memory up to n = 240, else in L2 with the pairs
-//      spread over a cluster of 8 SMs (its hardware barrier costs a fraction of a launch).
+//      definite, so its columns converge to lambda_j v_j and need no second matrix.  One warp per column pair, the
+//      whole matrix in one SM's shared memory.
 //   2. Two passes of the iterative refinement of the symmetric eigendecomposition (T. Ogita and K. Aishima, Japan J.
 //      Indust. Appl. Math. 35, 2018): R = I - X^T X, S = X^T A X, X += X E with E_ij = (s_ij + l_j r_ij) / (l_j - l_i),
 //      or r_ij / 2 for eigenvalues closer than 1e-4 (second pass: 1e-8) of the spectrum's RMS, where the quotient
@@ -376,9 +374,11 @@ __global__ void k_drop_index(int m, int* perm, int x)
 // clustered ones (one or two).
 // An eigenvector's sign (and a basis of an exactly degenerate space) is whatever the method happens to give:
 // hf_eigh, whose eigenvectors the caller sees, keeps the plain Jacobi start and with it its signs; the SCF, which
-// only uses the density they span, starts here (EighStart).  Measured in a 4-water SCF (n = 100, 11
+// only uses the density they span, starts here (EighStart) up to the size that fits one SM.  Beyond it (the matrix in
+// L2, the pairs over a cluster of 8 SMs) the phase took longer than the four or five sweeps that a start from the last
+// iteration's eigenvectors leaves: n = 800 0.17 s a diagonalisation against 0.125 s.  Measured in a 4-water SCF (n = 100, 11
 // diagonalisations): 29 ms of Jacobi kernels and their launch gaps before, 12.5 ms with this start.
-constexpr int kPre32MinN = 4, kPre32MaxN = 2048, kPre32SmemN = 240;
+constexpr int kPre32MinN = 4, kPre32MaxN = 240;
 constexpr int kPre32Sweeps = 15;
 
 // scale[0] = max |a_ij|, scale[1] = max row sum of |a_ij|
@@ -437,43 +437,32 @@ __device__ __forceinline__ float warp_sum(float v)
     return v;
 }
 
-// One-sided Jacobi sweeps on the n columns of G (column j at G + j n).  NC: elements of a column per lane.
-// SMEM: one block, G copied to shared memory; else the blocks of one cluster share G in global memory.
-template <int NC, int NT, bool SMEM>
-__device__ __forceinline__ void pre_sweeps(int n, float* __restrict__ Gg, int* __restrict__ flags)
+// One-sided Jacobi sweeps on the n <= 240 columns of G (column j at G + j n), eight elements of a column per lane.
+__global__ void __launch_bounds__(1024) k_pre_sweeps(int n, float* __restrict__ Gg)
 {
-    namespace cg = cooperative_groups;
-    extern __shared__ float gsh[];
+    constexpr int NC = (kPre32MaxN + 31) / 32;
+    extern __shared__ float G[];
     __shared__ int changed;
-    float* const G = SMEM ? gsh : Gg;
-    const int lane = threadIdx.x & 31, nblk = SMEM ? 1 : (int)gridDim.x;
-    const int warp = (threadIdx.x >> 5) * nblk + (SMEM ? 0 : (int)blockIdx.x), nwarps = (NT >> 5) * nblk;
-    auto barrier = [&]() {
-        if constexpr (SMEM)
-            __syncthreads();
-        else
-            cg::this_cluster().sync();
-    };
-    if (SMEM)
-        for (int e = threadIdx.x; e < n * n; e += NT) G[e] = Gg[e];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int e = threadIdx.x; e < n * n; e += 1024) G[e] = Gg[e];
     const int m = n + (n & 1);
     for (int sweep = 0; sweep < kPre32Sweeps; sweep++) {
         if (threadIdx.x == 0) changed = 0;
-        barrier();
+        __syncthreads();
         for (int r = 0; r < m - 1; r++) {
-            for (int k = warp; k < m / 2; k += nwarps) {
+            for (int k = warp; k < m / 2; k += 32) {
                 int p, q;
                 rr_pair(m, r, k, p, q);
                 if (p >= n || q >= n) continue;  // the padding index of an odd n
-                float* const gp = G + (size_t)p * n;
-                float* const gq = G + (size_t)q * n;
+                float* const gp = G + p * n;
+                float* const gq = G + q * n;
                 float x[NC], y[NC];
                 float aa = 0.0f, bb = 0.0f, ab = 0.0f;
 #pragma unroll
                 for (int i = 0; i < NC; i++) {
                     const int e = lane + 32 * i;
-                    x[i] = e < n ? (SMEM ? gp[e] : __ldcg(gp + e)) : 0.0f;
-                    y[i] = e < n ? (SMEM ? gq[e] : __ldcg(gq + e)) : 0.0f;
+                    x[i] = e < n ? gp[e] : 0.0f;
+                    y[i] = e < n ? gq[e] : 0.0f;
                     aa = fmaf(x[i], x[i], aa);
                     bb = fmaf(y[i], y[i], bb);
                     ab = fmaf(x[i], y[i], ab);
@@ -492,41 +481,18 @@ __device__ __forceinline__ void pre_sweeps(int n, float* __restrict__ Gg, int* _
                 for (int i = 0; i < NC; i++) {
                     const int e = lane + 32 * i;
                     if (e < n) {
-                        const float u = c * x[i] - s * y[i], v = s * x[i] + c * y[i];
-                        if (SMEM) {
-                            gp[e] = u;
-                            gq[e] = v;
-                        } else {
-                            __stcg(gp + e, u);
-                            __stcg(gq + e, v);
-                        }
+                        gp[e] = c * x[i] - s * y[i];
+                        gq[e] = s * x[i] + c * y[i];
                     }
                 }
             }
-            barrier();
-        }
-        bool any;
-        if constexpr (SMEM) {
-            any = changed != 0;
             __syncthreads();
-        } else {
-            if (threadIdx.x == 0 && changed) atomicOr(flags + sweep, 1);
-            barrier();
-            any = __ldcg(flags + sweep) != 0;
         }
+        const bool any = changed != 0;
+        __syncthreads();
         if (!any) break;
     }
-    if (SMEM)
-        for (int e = threadIdx.x; e < n * n; e += NT) Gg[e] = G[e];
-}
-
-__global__ void __launch_bounds__(1024) k_pre_smem(int n, float* __restrict__ G) { pre_sweeps<8, 1024, true>(n, G, nullptr); }
-
-template <int NC, int NT>
-__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(NT) k_pre_cluster(int n, float* __restrict__ G,
-                                                                              int* __restrict__ flags)
-{
-    pre_sweeps<NC, NT, false>(n, G, flags);
+    for (int e = threadIdx.x; e < n * n; e += 1024) Gg[e] = G[e];
 }
 
 // X[:, j] = g_j / |g_j| (one warp per column), X row-major
@@ -596,23 +562,13 @@ __global__ void k_schulz(int n, double* __restrict__ Q)
 static int pre_eigenbasis(int n, const double* As, double*& X, double*& T, double* S, double* Q, float* G, double* part,
                           double* scal, cudaStream_t s)
 {
-    const unsigned long long* scale = (const unsigned long long*)scal;  // 2 words, 16 flags, then lambda
-    int* flags = (int*)(scal + 2);
-    double* lam = scal + 10;
+    const unsigned long long* scale = (const unsigned long long*)scal;  // 2 words, then lambda
+    double* lam = scal + 2;
     const unsigned nb = (unsigned)(((long long)n * n + 255) / 256);
     k_pre_shift<<<nb, 256, 0, s>>>(n, As, scale, G);
-    if (n <= kPre32SmemN) {
-        const int bytes = n * n * (int)sizeof(float);
-        if (cudaFuncSetAttribute(k_pre_smem, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kPre32SmemN * kPre32SmemN * (int)sizeof(float)) != cudaSuccess) return -1;
-        k_pre_smem<<<1, 1024, bytes, s>>>(n, G);
-    } else if (n <= 512) {
-        k_pre_cluster<16, 1024><<<8, 1024, 0, s>>>(n, G, flags);
-    } else if (n <= 1024) {
-        k_pre_cluster<32, 512><<<8, 512, 0, s>>>(n, G, flags);
-    } else {
-        k_pre_cluster<64, 256><<<8, 256, 0, s>>>(n, G, flags);
-    }
+    if (cudaFuncSetAttribute(k_pre_sweeps, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kPre32MaxN * kPre32MaxN * (int)sizeof(float)) != cudaSuccess) return -1;
+    k_pre_sweeps<<<1, 1024, n * n * (int)sizeof(float), s>>>(n, G);
     k_pre_normalise<<<(n + 7) / 8, 256, 0, s>>>(n, G, X);
     for (int it = 0; it < 4; it++) {
         if (gemm(n, n, n, 1.0, X, n, true, X, n, false, 0.0, Q, n, s)) return -1;
@@ -659,9 +615,9 @@ int jacobi_eigh(int n, const double* Ain, double* w, double* Vout, int ncols, do
     double* X = As + mm;
     double* T = X + mm;
     double* scal = T + mm;
-    float* G = (float*)(scal + 16 + m);
+    float* G = (float*)(scal + 2 + m);
     unsigned long long* scale = (unsigned long long*)scal;
-    if (cudaMemsetAsync(scal, 0, sizeof(double) * 10, s) != cudaSuccess) return -1;
+    if (cudaMemsetAsync(scal, 0, sizeof(double) * 2, s) != cudaSuccess) return -1;
     k_pre_norms<<<n, 256, 0, s>>>(n, Ain, scale);
     k_symmetrise<<<(unsigned)(((long long)n * n + 255) / 256), 256, 0, s>>>(n, Ain, scale, As);
     double* cur = A0;
@@ -915,8 +871,8 @@ namespace hf {
 size_t jacobi_work_doubles(int n)
 {
     const size_t m = (size_t)(n + (n & 1));
-    // As, X, T; norms, flags, sums and lambda; G in FP32
-    return jacobi_work_base(n) + 3 * m * m + 16 + m + (m * m + 1) / 2;
+    // As, X, T; norms and lambda; G in FP32
+    return jacobi_work_base(n) + 3 * m * m + 2 + m + (m * m + 1) / 2;
 }
 size_t jacobi_work_ints(int n)
 {

@@ -125,8 +125,7 @@ __device__ __forceinline__ void one_electron_pair(const OneEArgs& a, int pid, do
         for (int i = 0; i < C::NR; i++) RS[i] = 0.0;
         for (int nuc = nslot; nuc < a.n_atoms; nuc += gn)
             C::nucleus(bp, a.xyz[3 * nuc], a.xyz[3 * nuc + 1], a.xyz[3 * nuc + 2], a.Z[nuc], a.boys64, RS);
-        // record prefactor sqrt(2) pi^(5/4) / p ... -> -2 pi / p ...
-        C::scale(bp, -1.0622519320271969 * bp.K, RS, acc);  // sqrt(2) pi^(-1/4)
+        C::scale(bp, -kNuclearPrefactor * bp.K, RS, acc);  // the record's sqrt(2) pi^(5/4) / p to -2 pi / p
     }
 #pragma unroll
     for (int i = 0; i < C::NI; i++)

@@ -164,7 +164,6 @@ __global__ void k_build_pairs(long long n_pairs, int maxpp, const int* __restric
     h.ABfz = (float)ABz;
     pairs[t] = h;
     pclass[t] = la * (la + 1) / 2 + lb;
-    const double c52 = sqrt(2.0) * pow(M_PI, 1.25);  // sqrt(2) pi^(5/4)
     int k = 0;
     for (int ka = 0; ka < nprim[A]; ka++) {
         const double a = exps[prim0[A] + ka], ca = cn[prim0[A] + ka];
@@ -179,7 +178,7 @@ __global__ void k_build_pairs(long long n_pairs, int maxpp, const int* __restric
             r.PAx = r.Px - Ax;
             r.PAy = r.Py - Ay;
             r.PAz = r.Pz - Az;
-            r.K = ca * cb * exp(-a * b * ip * R2) * c52 * ip;
+            r.K = ca * cb * exp(-a * b * ip * R2) * kPairPrefactor * ip;
             r.oo2p = 0.5 * ip;
             r.B = 0.0f;  // set by the Schwarz pass; 0 never stops a primitive loop whose threshold is 0
             p64[t * maxpp + k] = r;
@@ -187,10 +186,13 @@ __global__ void k_build_pairs(long long n_pairs, int maxpp, const int* __restric
             q.Px = r.Px;
             q.Py = r.Py;
             q.Pz = r.Pz;
-            q.K = r.K;
-            for (int x = 0; x < la + lb; x++) q.K *= r.oo2p;
             q.u = 2.0 * b;
             q.v = 2.0 * p;
+            // K (2p)^-W by one division: the scalings multiply it by powers of the same 2p, and W factors of a rounded
+            // 1/(2p) would leave W times its error in every integral of the pair
+            double pw = p;
+            for (int x = 0; x < la + lb; x++) pw *= q.v;
+            q.K = ca * cb * exp(-a * b * ip * R2) * kPairPrefactor / pw;
             const int ta = utype[prim0[A] + ka], tb = utype[prim0[B] + kb];
             q.type = max(ta, tb) * (max(ta, tb) + 1) / 2 + min(ta, tb);
             q.pad[0] = q.pad[1] = q.pad[2] = 0;

@@ -304,7 +304,7 @@ class System:
         timed call) or a CUDA float64 tensor (device path).  Output buffers may
         be passed to avoid allocation.  rys: True for Rys quadrature in all five
         L >= 6 classes (HF_RYS), False for Obara-Saika in every class
-        (HF_OBARA_SAIKA), None for the per-class default.  Returns a dict with
+        (HF_OBARA_SAIKA), None for the default (Hermite accumulators).  Returns a dict with
         F, J, K, E_elec and optionally stats."""
         N = self.n_bf
         lib = load_library()
@@ -536,7 +536,7 @@ def _is_dev(x) -> bool:
 
 
 def _method_flags(rys) -> int:
-    """ERI method flags: True -> HF_RYS, False -> HF_OBARA_SAIKA, None -> 0 (the per-class default)."""
+    """ERI method flags: True -> HF_RYS, False -> HF_OBARA_SAIKA, None -> 0 (Hermite accumulators)."""
     return 0 if rys is None else (HF_RYS if rys else HF_OBARA_SAIKA)
 
 
