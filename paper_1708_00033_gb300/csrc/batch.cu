@@ -272,7 +272,11 @@ int hf_batch_create(hf_ctx* ctx, int n_mol, const hf_geometry* geoms, const hf_b
     if ((rc = B->counters.alloc(sizeof(unsigned long long) * kNumClasses)) != HF_OK) return cleanup(rc);
     if (cudaStreamCreateWithFlags(&B->st, cudaStreamNonBlocking) != cudaSuccess)
         return cleanup(cuda_status(cudaGetLastError(), "hf_batch: stream"));
-    cudaEventCreateWithFlags(&B->fork, cudaEventDisableTiming);
+    // create_system returns with its last kernels (pair headers, tables) in flight on the context's stream; everything
+    // on this batch's own stream, graph launches and tuning included, comes after them
+    if (cudaEventCreateWithFlags(&B->fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventRecord(B->fork, ctx->stream) != cudaSuccess || cudaStreamWaitEvent(B->st, B->fork, 0) != cudaSuccess)
+        return cleanup(cuda_status(cudaGetLastError(), "hf_batch: order after the set-up"));
     cudaEventCreate(&B->t0);
     cudaEventCreate(&B->t1);
     cudaMemcpyAsync(B->eoff.p, B->eoff_h.data(), sizeof(long long) * (n_mol + 1), cudaMemcpyHostToDevice, B->st);
