@@ -138,6 +138,7 @@ struct hf_batch {
     cudaStream_t st = nullptr;
     cudaStream_t cst[kNumClasses] = {};
     cudaEvent_t fork = nullptr, join[kNumClasses] = {}, t0 = nullptr, t1 = nullptr;
+    cudaEvent_t ready = nullptr;  // the context's stream, when work on `st` begins
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     int num_sms = 0;
@@ -150,6 +151,7 @@ struct hf_batch {
             if (join[c]) cudaEventDestroy(join[c]);
         }
         if (fork) cudaEventDestroy(fork);
+        if (ready) cudaEventDestroy(ready);
         if (t0) cudaEventDestroy(t0);
         if (t1) cudaEventDestroy(t1);
         if (st) cudaStreamDestroy(st);
@@ -275,7 +277,8 @@ int hf_batch_create(hf_ctx* ctx, int n_mol, const hf_geometry* geoms, const hf_b
     // create_system returns with its last kernels (pair headers, tables) in flight on the context's stream; everything
     // on this batch's own stream, graph launches and tuning included, comes after them
     if (cudaEventCreateWithFlags(&B->fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventRecord(B->fork, ctx->stream) != cudaSuccess || cudaStreamWaitEvent(B->st, B->fork, 0) != cudaSuccess)
+        cudaEventCreateWithFlags(&B->ready, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventRecord(B->ready, ctx->stream) != cudaSuccess || cudaStreamWaitEvent(B->st, B->ready, 0) != cudaSuccess)
         return cleanup(cuda_status(cudaGetLastError(), "hf_batch: order after the set-up"));
     cudaEventCreate(&B->t0);
     cudaEventCreate(&B->t1);
@@ -374,6 +377,11 @@ int hf_fock_build_batch(hf_batch* B, const double* P, double* F, double* E_elec,
         HF_CUDA(cudaEventSynchronize(B->t1));
         if (ms) cudaEventElapsedTime(ms, B->t0, B->t1);
         return HF_OK;
+    }
+    // the caller's pending work on the context's stream may still write P or read F
+    if (dev) {
+        HF_CUDA(cudaEventRecord(B->ready, B->ctx->stream));
+        HF_CUDA(cudaStreamWaitEvent(st, B->ready, 0));
     }
     HF_CUDA(cudaMemcpyAsync(B->Pin.p, P, bytes, dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
     HF_CUDA(cudaEventRecord(B->t0, st));

@@ -54,6 +54,8 @@ void rec_read_words(int on, unsigned long long word)               // copies to 
     g_word = word;
 }
 
+void rec_launch(unsigned long long stream, const char* name) { log("launch", (void*)stream, name); }  // the caller's own
+
 // -------------------------------------------------------------- the runtime --
 void** __cudaRegisterFatBinary(void*) { return (void**)handle(); }
 void __cudaRegisterFatBinaryEnd(void**) {}

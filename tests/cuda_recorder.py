@@ -34,6 +34,7 @@ def recorded(stream: int = 8):
             lib.rec_log.restype = ctypes.c_char_p
             lib.rec_live_bytes.restype = lib.rec_peak_bytes.restype = ctypes.c_ulonglong
             lib.rec_set_limit.argtypes = [ctypes.c_ulonglong]
+            lib.rec_launch.argtypes = [ctypes.c_ulonglong, ctypes.c_char_p]
             lib.rec_read_words.argtypes = [ctypes.c_int, ctypes.c_ulonglong]
             ctx = hf.Context(0, stream=stream)
             try:
