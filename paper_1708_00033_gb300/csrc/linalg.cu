@@ -338,7 +338,7 @@ __global__ void k_gather_eig(int n, int m, int ncols, const double* __restrict__
 
 int bitonic_sort_desc(double* key, int* val, int n, int n_pad, cudaStream_t s);
 
-// doubles of the Jacobi sweeps' own workspace: A, its ping-pong copy and V, partial sums, sort keys
+// doubles of the Jacobi sweeps' own workspace: A, its ping-pong copy and V, partial sums, sort keys, norms and lambda
 static size_t jacobi_work_base(int n)
 {
     const size_t m = (size_t)(n + (n & 1));
@@ -379,6 +379,10 @@ __global__ void k_drop_index(int m, int* perm, int x)
 // iteration's eigenvectors leaves: n = 800 0.17 s a diagonalisation against 0.125 s.  Measured in a 4-water SCF (n = 100, 11
 // diagonalisations): 29 ms of Jacobi kernels and their launch gaps before, 12.5 ms with this start.
 constexpr int kPre32MinN = 4, kPre32MaxN = 240;
+static bool uses_basis32(int n, EighStart start)
+{
+    return start == EighStart::kBasis32 && n >= kPre32MinN && n <= kPre32MaxN;
+}
 constexpr int kPre32Sweeps = 15;
 
 // scale[0] = max |a_ij|, scale[1] = max row sum of |a_ij|
@@ -601,7 +605,7 @@ __global__ void k_gather_cols(int n, int ncols, const double* __restrict__ X, co
 int jacobi_eigh(int n, const double* Ain, double* w, double* Vout, int ncols, double* work, int* iwork, int max_sweeps,
                 double tol, EighStart start, int* sweeps_done, cudaStream_t s)
 {
-    // work: jacobi_work_doubles(n) doubles; iwork: m_pad ints
+    // work: jacobi_work_doubles(n, start) doubles; iwork: m_pad ints
     const int m = n + (n & 1);
     if (n <= 0) return 0;
     const size_t mm = (size_t)m * m;
@@ -611,11 +615,15 @@ int jacobi_eigh(int n, const double* Ain, double* w, double* Vout, int ncols, do
     double* part = V + mm;
     double* res = part + 512;
     double* key = res + 2;
-    double* As = work + jacobi_work_base(n);
+    size_t mp = 1;
+    while (mp < (size_t)m) mp <<= 1;
+    double* scal = key + mp;  // two norms, then lambda
+    // the FP32 start keeps A beside its products (As, X, T; G in FP32); otherwise A is read once, from A1
+    bool pre = uses_basis32(n, start);
+    double* As = pre ? work + jacobi_work_base(n) : A1;
     double* X = As + mm;
     double* T = X + mm;
-    double* scal = T + mm;
-    float* G = (float*)(scal + 2 + m);
+    float* G = (float*)(T + mm);
     unsigned long long* scale = (unsigned long long*)scal;
     if (cudaMemsetAsync(scal, 0, sizeof(double) * 2, s) != cudaSuccess) return -1;
     k_pre_norms<<<n, 256, 0, s>>>(n, Ain, scale);
@@ -632,7 +640,6 @@ int jacobi_eigh(int n, const double* Ain, double* w, double* Vout, int ncols, do
     };
     // The Jacobi sweeps start from S = X^T A X (in A1) when X came out orthonormal (a matrix that is not finite, or an
     // FP32 phase that did not converge, shows here), else from A itself.
-    bool pre = start == EighStart::kBasis32 && n >= kPre32MinN && n <= kPre32MaxN;
     if (pre) {
         if (pre_eigenbasis(n, As, X, T, A1, V, G, part, scal, s)) return -1;
         if (off_norms(n, V)) return -1;  // Q = X^T X: off-diagonal part and sum of squares (n for the identity)
@@ -653,8 +660,6 @@ int jacobi_eigh(int n, const double* Ain, double* w, double* Vout, int ncols, do
         if (cudaGetLastError() != cudaSuccess) return -1;
     }
     if (sweeps_done) *sweeps_done = sweep;
-    size_t mp = 1;
-    while (mp < (size_t)m) mp <<= 1;
     k_diag_keys<<<(unsigned)((mp + 255) / 256), 256, 0, s>>>(m, cur, key, iwork, (int)mp);
     if (bitonic_sort_desc(key, iwork, (int)mp, (int)mp, s) != 0) return -1;
     // when n is odd the padding index m-1 carries eigenvalue 0 and must be skipped: drop it from perm
@@ -868,11 +873,10 @@ int scale_cols(int n, int ncols, const double* U, const double* s, double power,
 }  // namespace hf
 
 namespace hf {
-size_t jacobi_work_doubles(int n)
+size_t jacobi_work_doubles(int n, EighStart start)
 {
     const size_t m = (size_t)(n + (n & 1));
-    // As, X, T; norms and lambda; G in FP32
-    return jacobi_work_base(n) + 3 * m * m + 2 + m + (m * m + 1) / 2;
+    return jacobi_work_base(n) + (uses_basis32(n, start) ? 3 * m * m + (m * m + 1) / 2 : 0);  // As, X, T; G in FP32
 }
 size_t jacobi_work_ints(int n)
 {

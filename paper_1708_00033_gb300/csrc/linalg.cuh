@@ -8,14 +8,14 @@ int gemm(int M, int N, int K, double alpha, const double* A, int lda, bool ta, c
          double beta, double* C, int ldc, cudaStream_t s);
 // Eigen-decomposition of a symmetric n x n matrix by parallel cyclic Jacobi.
 // w[ncols]: lowest ncols eigenvalues ascending; Vout[n x ncols] the matching
-// eigenvectors as columns.  work: jacobi_work_doubles(n) doubles, iwork: jacobi_work_ints(n) ints.
+// eigenvectors as columns.  work: jacobi_work_doubles(n, start) doubles, iwork: jacobi_work_ints(n) ints.
 // start: where the FP64 sweeps start, the matrix itself or an FP32 eigenbasis refined in FP64 (fewer or no sweeps
 // left; the eigenvectors' signs then follow that basis).
 // Returns 0 converged, 1 not converged within max_sweeps, -1 CUDA error.
 enum class EighStart { kMatrix, kBasis32 };
 int jacobi_eigh(int n, const double* A, double* w, double* Vout, int ncols, double* work, int* iwork, int max_sweeps,
                 double tol, EighStart start, int* sweeps_done, cudaStream_t s);
-size_t jacobi_work_doubles(int n);
+size_t jacobi_work_doubles(int n, EighStart start);
 size_t jacobi_work_ints(int n);
 int antisym(int n, const double* A, double* E, cudaStream_t s);
 int dots(long long len, const double* X, const double* const* Ys_dev, int nk, double* part, double* out,

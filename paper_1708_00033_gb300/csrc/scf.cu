@@ -58,14 +58,16 @@ double now_s()
 struct Eigh {
     DevBuf work, iwork;
     int n = 0;
-    int init(int n_)
+    EighStart start = EighStart::kMatrix;
+    int init(int n_, EighStart start_)
     {
         n = n_;
-        S_TRY(work.alloc(jacobi_work_doubles(n) * sizeof(double)));
+        start = start_;
+        S_TRY(work.alloc(jacobi_work_doubles(n, start) * sizeof(double)));
         S_TRY(iwork.alloc(jacobi_work_ints(n) * sizeof(int)));
         return HF_OK;
     }
-    int run(const double* A, double* w, double* V, int ncols, EighStart start, int* sweeps, cudaStream_t s)
+    int run(const double* A, double* w, double* V, int ncols, int* sweeps, cudaStream_t s)
     {
         int sw = 0;
         const int rc = jacobi_eigh(n, A, w, V, ncols, work.as<double>(), iwork.as<int>(), 60, 1e-14, start,
@@ -103,8 +105,8 @@ extern "C" int hf_eigh(hf_ctx* ctx, int n, const double* A, double* w, double* V
         pV = dV.as<double>();
     }
     Eigh e;
-    S_TRY(e.init(n));
-    S_TRY(e.run(pA, pw, pV, n, EighStart::kMatrix, nullptr, st));
+    S_TRY(e.init(n, EighStart::kMatrix));
+    S_TRY(e.run(pA, pw, pV, n, nullptr, st));
     if (!dev) {
         HF_CUDA(cudaMemcpyAsync(w, pw, n * sizeof(double), cudaMemcpyDeviceToHost, st));
         HF_CUDA(cudaMemcpyAsync(V, pV, nn * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -177,11 +179,11 @@ extern "C" int hf_scf_run(hf_system* S, const hf_scf_opts* opts_in, const double
         S_TRY(Eh[k].alloc(NN * sizeof(double)));
     }
     Eigh eig;
-    S_TRY(eig.init(N));
+    S_TRY(eig.init(N, EighStart::kBasis32));
     int sweeps = 0;
     double t_diag = 0.0, t_fock = 0.0;
     double td = now_s();
-    S_TRY(eig.run(S->S.as<double>(), sv.as<double>(), U.as<double>(), N, EighStart::kBasis32, &sweeps, st));
+    S_TRY(eig.run(S->S.as<double>(), sv.as<double>(), U.as<double>(), N, &sweeps, st));
     std::vector<double> s_host(N);
     HF_CUDA(cudaMemcpyAsync(s_host.data(), sv.p, N * sizeof(double), cudaMemcpyDeviceToHost, st));
     HF_CUDA(cudaStreamSynchronize(st));
@@ -220,7 +222,7 @@ extern "C" int hf_scf_run(hf_system* S, const hf_scf_opts* opts_in, const double
         Eigh* e = &eig;
         Eigh e2;
         if (nx != N) {
-            rc = e2.init(nx);
+            rc = e2.init(nx, EighStart::kBasis32);
             if (rc != HF_OK) return rc;
             e = &e2;
         }
@@ -231,13 +233,13 @@ extern "C" int hf_scf_run(hf_system* S, const hf_scf_opts* opts_in, const double
             if (gemm(nx, nx, nx, 1.0, Vprev.as<double>(), nx, true, T1.as<double>(), nx, false, 0.0, Fw.as<double>(),
                      nx, st))
                 return -1;
-            rc = e->run(Fw.as<double>(), eps, Vj.as<double>(), nx, EighStart::kBasis32, &sweeps, st);
+            rc = e->run(Fw.as<double>(), eps, Vj.as<double>(), nx, &sweeps, st);
             if (rc != HF_OK) return rc;
             if (gemm(nx, nx, nx, 1.0, Vprev.as<double>(), nx, false, Vj.as<double>(), nx, false, 0.0, Vp.as<double>(),
                      nx, st))
                 return -1;
         } else {
-            rc = e->run(Fp.as<double>(), eps, Vp.as<double>(), nx, EighStart::kBasis32, &sweeps, st);
+            rc = e->run(Fp.as<double>(), eps, Vp.as<double>(), nx, &sweeps, st);
             if (rc != HF_OK) return rc;
         }
         if (cudaMemcpyAsync(Vprev.p, Vp.p, (size_t)nx * nx * sizeof(double), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
