@@ -317,10 +317,11 @@ __global__ void k_diag_keys(int m, const double* __restrict__ A, double* __restr
 
 // The matrix is worked on times this power of two (exact), which brings max |a_ij| into [1, 2): the sums of
 // squares of the convergence tests and the FP32 steps neither under- nor overflow.  scale[0] = bits of max |a_ij|.
+// Subnormal matrices take the largest power whose double is finite too (2^1022): they end up above 2^-52.
 __device__ __forceinline__ double eigh_factor(const unsigned long long* scale)
 {
     const double mx = __longlong_as_double(scale[0]);
-    return mx > 0.0 && isfinite(mx) ? ldexp(1.0, -ilogb(mx)) : 1.0;
+    return mx > 0.0 && isfinite(mx) ? ldexp(1.0, min(-ilogb(mx), 1022)) : 1.0;
 }
 
 // w[j] = lambda of sorted column j; Vout[:, j] = V[:n, perm[j]] for j < ncols
