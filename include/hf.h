@@ -345,7 +345,8 @@ int hf_scf_run(hf_system* sys, const hf_scf_opts* opts, const double* P_guess, d
  * cyclic Jacobi, the diagonalisation step of Section 3's SCF).  w[n]
  * eigenvalues ascending; V[n*n] row-major with eigenvector j in column j.
  * flags: HF_PTR_DEVICE for device pointers.  Errors: HF_E_INVALID,
- * HF_E_NOMEM, HF_E_CUDA, HF_E_NOCONV (60 sweeps). */
+ * HF_E_NOMEM, HF_E_CUDA, HF_E_NOCONV (60 sweeps, or A is not finite; w and V
+ * are then not meaningful). */
 int hf_eigh(hf_ctx* ctx, int n, const double* A, double* w, double* V, int flags);
 
 /* --------------------------------------------------------------- batches */

@@ -652,6 +652,9 @@ int jacobi_eigh(int n, const double* Ain, double* w, double* Vout, int ncols, do
     int sweep = 0;
     for (sweep = 0; sweep < max_sweeps; sweep++) {
         if (off_norms(m, cur)) return -1;
+        // A is scaled, so its norm overflows only if an element was infinite or NaN: no eigenpairs, and no sort of NaN
+        // keys, which would bring the padding's index (0x7fffffff) into the permutation
+        if (!isfinite(h[1])) return 1;
         if (h[0] <= tol * tol * h[1] || h[0] == 0.0) break;
         for (int r = 0; r < m - 1; r++) {
             // every entry of Anew belongs to exactly one (row pair, column pair) block of this round

@@ -11,7 +11,8 @@ int gemm(int M, int N, int K, double alpha, const double* A, int lda, bool ta, c
 // eigenvectors as columns.  work: jacobi_work_doubles(n, start) doubles, iwork: jacobi_work_ints(n) ints.
 // start: where the FP64 sweeps start, the matrix itself or an FP32 eigenbasis refined in FP64 (fewer or no sweeps
 // left; the eigenvectors' signs then follow that basis).
-// Returns 0 converged, 1 not converged within max_sweeps, -1 CUDA error.
+// Returns 0 converged, 1 not converged within max_sweeps or A not finite (w and Vout are then not written),
+// -1 CUDA error.
 enum class EighStart { kMatrix, kBasis32 };
 int jacobi_eigh(int n, const double* A, double* w, double* Vout, int ncols, double* work, int* iwork, int max_sweeps,
                 double tol, EighStart start, int* sweeps_done, cudaStream_t s);

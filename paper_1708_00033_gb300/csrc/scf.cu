@@ -74,7 +74,7 @@ struct Eigh {
                                    &sw, s);
         if (sweeps) *sweeps += sw;
         if (rc < 0) return cuda_status(cudaGetLastError(), "jacobi_eigh");
-        if (rc > 0) return scf_fail(HF_E_NOCONV, "Jacobi eigensolver did not converge in 60 sweeps");
+        if (rc > 0) return scf_fail(HF_E_NOCONV, "Jacobi eigensolver: not converged in 60 sweeps, or the matrix is not finite");
         return HF_OK;
     }
 };

@@ -19,3 +19,22 @@ def test_eigh_extreme_scales(n, k):
     assert np.abs(np.ldexp(w, -k) - np.linalg.eigvalsh(B)).max() <= (2e-14 + n * eps) * norm + grid
     assert np.linalg.norm(V.T @ V - np.eye(n)) <= 13 * n * eps
     assert np.linalg.norm(B @ V - V * np.ldexp(w, -k)) <= (2e-14 + n * eps) * norm + grid * np.sqrt(n)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 8, 13, 40])
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("at", ["first", "last", "all"])
+def test_eigh_rejects_a_matrix_that_is_not_finite(n, bad, at):
+    """No eigenpairs and no answer; the context stays usable.  (The sort of NaN keys used to bring the index that pads
+    it to a power of two into the permutation of the gathered columns.)"""
+    from paper_1708_00033_gb300 import hf
+    ctx = hf.Context(0)
+    A = np.eye(n) + 0.01
+    i = slice(None) if at == "all" else 0 if at == "first" else n - 1
+    B = A.copy()
+    B[i, i] = bad
+    with pytest.raises(hf.HFError) as e:
+        hf.eigh(ctx, B)
+    assert e.value.code == hf.HF_E_NOCONV
+    w, _ = hf.eigh(ctx, A)
+    assert np.abs(w - np.linalg.eigvalsh(A)).max() <= 1e-13 * (1 + 0.01 * n)
