@@ -261,6 +261,12 @@ int create_system(hf_ctx* ctx, const hf_geometry* geom, const hf_basis* basis, c
 
 }  // namespace hf
 
+// hf_eigh of host arrays with the start that the SCF's diagonalisations take (EighStart::kBasis32); basis_used and sweeps
+// (nullable) tell whether the basis was accepted and how many sweeps it left.  Not part of the public interface: its
+// eigenvectors' signs follow the basis.
+extern "C" int hf_eigh_basis32(hf_ctx* ctx, int n, const double* A, double* w, double* V, int32_t* basis_used,
+                               int32_t* sweeps);
+
 // ----------------------------------------------------------- C-ABI types --
 struct hf_ctx {
     int device = 0;

@@ -369,10 +369,13 @@ __global__ void k_drop_index(int m, int* perm, int x)
 //   2. Two passes of the iterative refinement of the symmetric eigendecomposition (T. Ogita and K. Aishima, Japan J.
 //      Indust. Appl. Math. 35, 2018): R = I - X^T X, S = X^T A X, X += X E with E_ij = (s_ij + l_j r_ij) / (l_j - l_i),
 //      or r_ij / 2 for eigenvalues closer than 1e-4 (second pass: 1e-8) of the spectrum's RMS, where the quotient
-//      would be noise.
-//   3. Two Newton-Schulz steps X = X (3 I - X^T X) / 2 make X orthonormal to rounding.
-// Then off(X^T A X) is near 1e-15 |A| for separated eigenvalues (no Jacobi sweep) and below 1e-8 |A| for
-// clustered ones (one or two).
+//      would be noise, and where the quotient exceeds kPreMaxTurn.  The FP32 phase resolves eigenvectors to 1e-7 of the
+//      norm over the gap, so pairs with gaps below about 1e-5 ask for turns that a first-order step cannot make.
+//   3. Two Newton-Schulz steps X = X (3 I - X^T X) / 2 make X orthonormal to rounding: g turns E in a column leave
+//      d = g E^2, two steps take that to 0.4 d^4, which is 3e-15 for 20 turns of the largest E allowed.
+// Then off(X^T A X) is near 1e-15 |A| for separated eigenvalues (no Jacobi sweep) and below 1e-5 |A| where some pairs
+// were left alone (up to five sweeps, measured on groups of four).  Without the limit on E, matrices with groups of
+// eigenvalues 1e-8 to 1e-4 apart lost X's orthonormality and with it everything done here: the sweeps then start from A.
 // An eigenvector's sign (and a basis of an exactly degenerate space) is whatever the method happens to give:
 // hf_eigh, whose eigenvectors the caller sees, keeps the plain Jacobi start and with it its signs; the SCF, which
 // only uses the density they span, starts here (EighStart) up to the size that fits one SM.  Beyond it (the matrix in
@@ -385,6 +388,7 @@ static bool uses_basis32(int n, EighStart start)
     return start == EighStart::kBasis32 && n >= kPre32MinN && n <= kPre32MaxN;
 }
 constexpr int kPre32Sweeps = 15;
+constexpr double kPreMaxTurn = 1.0 / 256;
 
 // scale[0] = max |a_ij|, scale[1] = max row sum of |a_ij|
 __global__ void __launch_bounds__(256) k_pre_norms(int n, const double* __restrict__ A, unsigned long long* __restrict__ scale)
@@ -552,8 +556,9 @@ __global__ void k_refine_correction(int n, int nb, double guard, const double* _
     if (e >= (long long)n * n) return;
     const int i = (int)(e / n), j = (int)(e % n);
     const double r = (i == j ? 1.0 : 0.0) - Q[e];
-    const double d = lam[j] - lam[i];
-    Q[e] = (i == j ? 1.0 : 0.0) + (i != j && fabs(d) > close ? (S[e] + lam[j] * r) / d : 0.5 * r);
+    const double d = lam[j] - lam[i], t = S[e] + lam[j] * r;
+    const bool turn = i != j && fabs(d) > close && fabs(t) <= kPreMaxTurn * fabs(d);
+    Q[e] = (i == j ? 1.0 : 0.0) + (turn ? t / d : 0.5 * r);
 }
 
 // Q = X^T X -> (3 I - Q) / 2
@@ -604,7 +609,7 @@ __global__ void k_gather_cols(int n, int ncols, const double* __restrict__ X, co
 }
 
 int jacobi_eigh(int n, const double* Ain, double* w, double* Vout, int ncols, double* work, int* iwork, int max_sweeps,
-                double tol, EighStart start, int* sweeps_done, cudaStream_t s)
+                double tol, EighStart start, int* sweeps_done, bool* basis_used, cudaStream_t s)
 {
     // work: jacobi_work_doubles(n, start) doubles; iwork: m_pad ints
     const int m = n + (n & 1);
@@ -647,6 +652,7 @@ int jacobi_eigh(int n, const double* Ain, double* w, double* Vout, int ncols, do
         const double lim = 4e-16 * n;
         pre = h[0] <= lim * lim && fabs(h[1] - n) <= lim * n;
     }
+    if (basis_used) *basis_used = pre;
     // padding eigenvalue: a zero-coupled padding entry only needs to be distinct and is dropped from the output.
     k_jacobi_init<<<nbm, 256, 0, s>>>(n, m, pre ? A1 : As, A0, V, 0.0);
     int sweep = 0;

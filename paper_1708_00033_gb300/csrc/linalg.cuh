@@ -11,11 +11,12 @@ int gemm(int M, int N, int K, double alpha, const double* A, int lda, bool ta, c
 // eigenvectors as columns.  work: jacobi_work_doubles(n, start) doubles, iwork: jacobi_work_ints(n) ints.
 // start: where the FP64 sweeps start, the matrix itself or an FP32 eigenbasis refined in FP64 (fewer or no sweeps
 // left; the eigenvectors' signs then follow that basis).
+// basis_used (nullable): whether the sweeps started from that basis (false where it does not apply or was rejected).
 // Returns 0 converged, 1 not converged within max_sweeps or A not finite (w and Vout are then not written),
 // -1 CUDA error.
 enum class EighStart { kMatrix, kBasis32 };
 int jacobi_eigh(int n, const double* A, double* w, double* Vout, int ncols, double* work, int* iwork, int max_sweeps,
-                double tol, EighStart start, int* sweeps_done, cudaStream_t s);
+                double tol, EighStart start, int* sweeps_done, bool* basis_used, cudaStream_t s);
 size_t jacobi_work_doubles(int n, EighStart start);
 size_t jacobi_work_ints(int n);
 int antisym(int n, const double* A, double* E, cudaStream_t s);

@@ -67,11 +67,11 @@ struct Eigh {
         S_TRY(iwork.alloc(jacobi_work_ints(n) * sizeof(int)));
         return HF_OK;
     }
-    int run(const double* A, double* w, double* V, int ncols, int* sweeps, cudaStream_t s)
+    int run(const double* A, double* w, double* V, int ncols, int* sweeps, cudaStream_t s, bool* basis_used = nullptr)
     {
         int sw = 0;
         const int rc = jacobi_eigh(n, A, w, V, ncols, work.as<double>(), iwork.as<int>(), 60, 1e-14, start,
-                                   &sw, s);
+                                   &sw, basis_used, s);
         if (sweeps) *sweeps += sw;
         if (rc < 0) return cuda_status(cudaGetLastError(), "jacobi_eigh");
         if (rc > 0) return scf_fail(HF_E_NOCONV, "Jacobi eigensolver: not converged in 60 sweeps, or the matrix is not finite");
@@ -84,7 +84,8 @@ struct Eigh {
 
 using namespace hf;
 
-extern "C" int hf_eigh(hf_ctx* ctx, int n, const double* A, double* w, double* V, int flags)
+static int eigh(hf_ctx* ctx, int n, const double* A, double* w, double* V, int flags, EighStart start, bool* basis_used,
+                int* sweeps)
 {
     if (!ctx || !A || !w || !V || n <= 0) return scf_fail(HF_E_INVALID, "hf_eigh: NULL argument or n <= 0");
     ScopedDevice g(ctx->device);
@@ -105,14 +106,30 @@ extern "C" int hf_eigh(hf_ctx* ctx, int n, const double* A, double* w, double* V
         pV = dV.as<double>();
     }
     Eigh e;
-    S_TRY(e.init(n, EighStart::kMatrix));
-    S_TRY(e.run(pA, pw, pV, n, nullptr, st));
+    S_TRY(e.init(n, start));
+    S_TRY(e.run(pA, pw, pV, n, sweeps, st, basis_used));
     if (!dev) {
         HF_CUDA(cudaMemcpyAsync(w, pw, n * sizeof(double), cudaMemcpyDeviceToHost, st));
         HF_CUDA(cudaMemcpyAsync(V, pV, nn * sizeof(double), cudaMemcpyDeviceToHost, st));
     }
     HF_CUDA(cudaStreamSynchronize(st));
     return HF_OK;
+}
+
+extern "C" int hf_eigh(hf_ctx* ctx, int n, const double* A, double* w, double* V, int flags)
+{
+    return eigh(ctx, n, A, w, V, flags, EighStart::kMatrix, nullptr, nullptr);
+}
+
+extern "C" int hf_eigh_basis32(hf_ctx* ctx, int n, const double* A, double* w, double* V, int32_t* basis_used,
+                               int32_t* sweeps)
+{
+    bool used = false;
+    int sw = 0;
+    const int rc = eigh(ctx, n, A, w, V, HF_PTR_HOST, EighStart::kBasis32, &used, &sw);
+    if (basis_used) *basis_used = used;
+    if (sweeps) *sweeps = sw;
+    return rc;
 }
 
 extern "C" int hf_scf_run(hf_system* S, const hf_scf_opts* opts_in, const double* P_guess, double* P_out,
