@@ -127,7 +127,6 @@ struct hf_batch {
     hf_ctx* ctx = nullptr;
     int device = 0;
     int n_mol = 0;
-    ExponentTable etab;  // shared by the molecules' systems: one table in L2 instead of one per molecule
     std::vector<hf_system*> sys;
     std::vector<long long> eoff_h;  // [n_mol + 1]
     long long len = 0;
@@ -236,14 +235,16 @@ int hf_batch_create(hf_ctx* ctx, int n_mol, const hf_geometry* geoms, const hf_b
     hf_thresholds t{};
     if (th) t = *th;
     t.fp32_cutoff = 0.0;  // the batched path is FP64 throughout
+    std::vector<double> exps;  // of all molecules: they share one exponent table in L2
     for (int m = 0; m < n_mol; m++) {
         if (int rc = check_geometry_basis(&geoms[m], &bases[m], &t)) return cleanup(rc);
-        B->etab.add(bases[m]);
+        add_exponents(exps, bases[m]);
     }
-    if (int rc = B->etab.build(ctx->stream)) return cleanup(rc);
+    std::shared_ptr<const ExponentTable> table;
+    if (int rc = exponent_table(ctx, std::move(exps), table)) return cleanup(rc);
     for (int m = 0; m < n_mol; m++) {
         hf_system* s = nullptr;
-        int rc = create_system(ctx, &geoms[m], &bases[m], &t, &B->etab, &s);
+        int rc = create_system(ctx, &geoms[m], &bases[m], &t, table, &s);
         if (rc != HF_OK) return cleanup(rc);
         B->sys.push_back(s);
     }

@@ -53,13 +53,30 @@ void DevBuf::release()
     owned = true;
 }
 
-void ExponentTable::add(const hf_basis& b)
+void add_exponents(std::vector<double>& exps, const hf_basis& b)
 {
     long long n = 0;
     for (int s = 0; s < b.n_shells; s++) n += b.nprim[s];
     exps.insert(exps.end(), b.exps, b.exps + n);
     std::sort(exps.begin(), exps.end());
     exps.erase(std::unique(exps.begin(), exps.end()), exps.end());
+}
+
+int exponent_table(hf_ctx* ctx, std::vector<double> exps, std::shared_ptr<const ExponentTable>& out)
+{
+    std::lock_guard<std::mutex> lock(ctx->tables_lock);
+    auto& all = ctx->tables;
+    all.erase(std::remove_if(all.begin(), all.end(), [](const auto& w) { return w.expired(); }), all.end());
+    for (const auto& w : all) {
+        out = w.lock();
+        if (out && out->exps == exps) return HF_OK;
+    }
+    auto t = std::make_shared<ExponentTable>();
+    t->exps = std::move(exps);
+    const int rc = t->build(ctx->stream);
+    out = rc == HF_OK ? t : nullptr;
+    if (rc == HF_OK) all.push_back(t);
+    return rc;
 }
 
 int ExponentTable::build(cudaStream_t s)
@@ -297,7 +314,7 @@ struct SideStreams {
     ~SideStreams() { join(); }
 };
 
-static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* basis, const ExponentTable* shared)
+static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* basis)
 {
     hf_ctx* ctx = S->ctx;
     cudaStream_t st = ctx->stream;
@@ -345,14 +362,15 @@ static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* b
     const size_t NN = (size_t)nbf * nbf;
 
     // exponent table and each primitive's place in it
-    if (!shared) {
-        S->etab.add(*basis);
-        TRY(S->etab.build(st));
-        shared = &S->etab;
+    if (!S->etab) {
+        std::vector<double> exps;
+        add_exponents(exps, *basis);
+        TRY(exponent_table(ctx, std::move(exps), S->etab));
     }
+    const ExponentTable* const table = S->etab.get();
     std::vector<int> utype(npr);
     for (int k = 0; k < npr; k++)
-        utype[k] = (int)(std::lower_bound(shared->exps.begin(), shared->exps.end(), basis->exps[k]) - shared->exps.begin());
+        utype[k] = (int)(std::lower_bound(table->exps.begin(), table->exps.end(), basis->exps[k]) - table->exps.begin());
 
     // ---------------------------------------------- inputs, matrices, pairs
     DevBuf utype_in;
@@ -407,7 +425,7 @@ static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* b
     HF_CUDA(cudaMemsetAsync(S->hB.p, 0, sizeof(float) * npairs * X.maxpp, st));
     S->herm.rec = S->hrec.as<HermPair>();
     S->herm.B = S->hB.as<float>();
-    S->herm = shared->view(S->herm);
+    S->herm = table->view(S->herm);
     KCHK(launch_shell_coef(ns, S->sh_l.as<int>(), S->sh_nprim.as<int>(), S->sh_prim0.as<int>(), S->sh_exp.as<double>(),
                            coef_in.as<double>(), S->sh_coef.as<double>(), st));
     KCHK(launch_comp_norm(ns, S->sh_l.as<int>(), S->sh_bf0.as<int>(), S->comp_norm.as<double>(), st));
@@ -665,7 +683,7 @@ static const hf_basis* expand_sp_shells(const hf_basis* b, ExpandedBasis& e)
 }
 
 int hf::create_system(hf_ctx* ctx, const hf_geometry* geom, const hf_basis* basis_in, const hf_thresholds* th,
-                      const ExponentTable* shared, hf_system** out)
+                      std::shared_ptr<const ExponentTable> table, hf_system** out)
 {
     TRY(check_geometry_basis(geom, basis_in, th));
     ExpandedBasis eb;
@@ -675,8 +693,9 @@ int hf::create_system(hf_ctx* ctx, const hf_geometry* geom, const hf_basis* basi
     S->ctx = ctx;
     S->device = ctx->device;
     S->stream = ctx->stream;
+    S->etab = std::move(table);
     if (th) S->th = *th;
-    int rc = system_setup(S, geom, basis, shared);
+    int rc = system_setup(S, geom, basis);
     if (rc != HF_OK) {
         cudaStreamSynchronize(ctx->stream);
         delete S;
@@ -730,7 +749,7 @@ int hf_system_get_info(const hf_system* S, hf_system_info* info)
     const DevBuf* bufs[] = {&S->sh_l, &S->sh_atom, &S->sh_bf0, &S->sh_nprim, &S->sh_prim0, &S->sh_exp, &S->sh_coef,
                             &S->atom_xyz, &S->atom_Z, &S->comp_norm, &S->pairs, &S->prims64, &S->prims32,
                             &S->pair_class, &S->S, &S->H, &S->P64, &S->P32, &S->Jt, &S->Kt, &S->F, &S->Ebuf,
-                            &S->Qall, &S->staging_P, &S->staging_out, &S->hrec, &S->hB, &S->etab.tab};
+                            &S->Qall, &S->staging_P, &S->staging_out, &S->hrec, &S->hB, &S->etab->tab};
     for (auto* b : bufs) bytes += b->bytes;
     for (int c = 0; c < kNumPairClasses; c++)
         bytes += S->class_ids[c].bytes + S->class_q[c].bytes + S->ket_tab[c].bytes + S->class_hdr[c].bytes;

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -241,7 +243,6 @@ struct ExponentTable {
     std::vector<double> exps;  // distinct, ascending
     DevBuf tab, psum;
     int ntype = 0;
-    void add(const hf_basis& b);
     int build(cudaStream_t s);
     HermView view(HermView h) const
     {
@@ -251,13 +252,22 @@ struct ExponentTable {
     }
 };
 
+// Adds a basis' exponents to a sorted list without repetitions.
+void add_exponents(std::vector<double>& exps, const hf_basis& b);
+
+// The context's table over these exponents: one that a live system or batch holds, or a new one (its kernel is issued
+// on the context's stream, as is all work that reads it or an event that orders that work).  A table takes 1.7 MB for
+// the water basis and up to 33 MB, a one-water system without it 0.3 MB: systems of one basis share it, and the last
+// owner frees it.
+int exponent_table(hf_ctx* ctx, std::vector<double> exps, std::shared_ptr<const ExponentTable>& out);
+
 // Status of hf_system_create's argument checks.
 int check_geometry_basis(const hf_geometry* g, const hf_basis* b, const hf_thresholds* th);
 
-// hf_system_create on a shared exponent table (nullptr: the system builds its own).  A shared table holds every
-// exponent of the basis and outlives the system.
+// hf_system_create on a given exponent table (nullptr: the context's over the basis' exponents), which holds every
+// exponent of the basis.
 int create_system(hf_ctx* ctx, const hf_geometry* geom, const hf_basis* basis, const hf_thresholds* th,
-                  const ExponentTable* shared, hf_system** out);
+                  std::shared_ptr<const ExponentTable> table, hf_system** out);
 
 }  // namespace hf
 
@@ -280,6 +290,8 @@ struct hf_ctx {
     cudaStream_t side[hf::kSideStreams] = {};  // class launches of one build run on these, forked from and
     cudaEvent_t fork = nullptr, join[hf::kSideStreams + 1] = {};  // joined to `stream` (launch_eri_classes)
     void* noalloc_scratch = nullptr;  // device address of hf_fock_build_noalloc's fixed scratch
+    std::mutex tables_lock;
+    std::vector<std::weak_ptr<const hf::ExponentTable>> tables;  // exponent_table: those that systems or batches hold
 };
 
 struct hf_system {
@@ -296,7 +308,7 @@ struct hf_system {
     int n_pairs_all = 0, n_prim_pairs = 0;
     hf::DevBuf pairs, prims64, prims32, pair_class;
     hf::DevBuf hrec, hB;          // HermPair records and bounds (HermView)
-    hf::ExponentTable etab;       // unless a batch's systems share one
+    std::shared_ptr<const hf::ExponentTable> etab;
     hf::HermView herm{};
     int class_count[hf::kNumPairClasses] = {};
     hf::DevBuf class_ids[hf::kNumPairClasses];  // sorted significant pair ids
