@@ -173,6 +173,9 @@ static BatchArgs batch_args(hf_batch* B, int c, long long limit)
     return a;
 }
 
+constexpr int kBatchBlock = 128, kBatchChunk = 256, kBatchBps = 4;  // chunk: one sorted window
+constexpr int kTuneFormat = 2;  // of the tuning file; raised with every change of the batched kernels or the columns
+
 // persistent grid: bps blocks per SM of the thread kernels, twice as many of the one-warp blocks
 static int batch_grid(const hf_batch* B, int c, int bps)
 {
@@ -314,9 +317,9 @@ int hf_batch_create(hf_ctx* ctx, int n_mol, const hf_geometry* geoms, const hf_b
         if (cudaStreamCreateWithFlags(&B->cst[c], cudaStreamNonBlocking) != cudaSuccess)
             return cleanup(cuda_status(cudaGetLastError(), "hf_batch: class stream"));
         cudaEventCreateWithFlags(&B->join[c], cudaEventDisableTiming);
-        B->block[c] = 128;
-        B->chunk[c] = 256;  // one sorted window
-        B->bps[c] = 4;
+        B->block[c] = kBatchBlock;
+        B->chunk[c] = kBatchChunk;
+        B->bps[c] = kBatchBps;
     }
     if (cudaStreamSynchronize(B->st) != cudaSuccess) return cleanup(cuda_status(cudaGetLastError(), "hf_batch: setup"));
     if ((rc = capture_graph(B)) != HF_OK) return cleanup(rc);
@@ -404,14 +407,18 @@ int hf_batch_tune(hf_batch* B, const char* cache_path, int64_t sample_quartets)
     if (!B) return bfail(HF_E_INVALID, "hf_batch_tune: NULL batch");
     BatchDevice g(B->device);
     cudaStream_t st = B->st;
-    // cached choices
+    // cached choices, of this format on this device only: choices made for other kernels or another GPU are noise here
+    cudaDeviceProp prop;
+    HF_CUDA(cudaGetDeviceProperties(&prop, B->device));
+    const std::string header = "# hf_batch_tune format " + std::to_string(kTuneFormat) + ", " + prop.name + "\n";
     bool have[kNumClasses] = {};
     if (cache_path) {
         FILE* f = fopen(cache_path, "r");
         if (f) {
-            char name[32];
+            char line[512], name[32];
             int bl, ch, bp;
-            while (fscanf(f, "%31s %d %d %d", name, &bl, &ch, &bp) == 4)
+            const bool ours = fgets(line, sizeof(line), f) && header == line;
+            while (ours && fscanf(f, "%31s %d %d %d", name, &bl, &ch, &bp) == 4)
                 for (int c = 0; c < kNumClasses; c++)
                     if (!strcmp(name, kEriClasses[c].name) && bl > 0 && bl <= 256 && ch > 0 && bp > 0 && bp <= 16) {
                         B->block[c] = bl;
@@ -422,9 +429,10 @@ int hf_batch_tune(hf_batch* B, const char* cache_path, int64_t sample_quartets)
             fclose(f);
         }
     }
-    const int blocks[] = {64, 128, 256};
-    const int chunks[] = {32, 128, 512};
-    const int bpss[] = {2, 4, 8};
+    // the defaults come first, so that a tie keeps them
+    const int blocks[] = {kBatchBlock, 64, 256};
+    const int chunks[] = {kBatchChunk, 32, 128, 512};
+    const int bpss[] = {kBatchBps, 2, 8};
     for (int c = 0; c < kNumClasses; c++) {
         if (have[c] || B->n_total[c] <= 0) continue;
         // sample about 2e10 algorithmic operations per candidate launch (a few ms), at most sample_quartets
@@ -433,9 +441,11 @@ int hf_batch_tune(hf_batch* B, const char* cache_path, int64_t sample_quartets)
         limit = std::max(2048LL, std::min(limit, sample_quartets > 0 ? (long long)sample_quartets : 2000000LL));
         float best = 1e30f;
         int best_bl = B->block[c], best_ch = B->chunk[c], best_bp = B->bps[c];
+        const bool warp = kEriClasses[c].batch_warp;  // one warp per block and groups of a fixed size: bps alone matters
         for (int bl : blocks)
             for (int ch : chunks)
                 for (int bp : bpss) {
+                    if (warp && (bl != kBatchBlock || ch != kBatchChunk)) continue;
                     BatchArgs a = batch_args(B, c, limit);
                     a.chunk = ch;
                     HF_CUDA(cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), st));
@@ -462,6 +472,7 @@ int hf_batch_tune(hf_batch* B, const char* cache_path, int64_t sample_quartets)
     if (cache_path) {
         FILE* f = fopen(cache_path, "w");
         if (f) {
+            fputs(header.c_str(), f);
             for (int c = 0; c < kNumClasses; c++)
                 fprintf(f, "%s %d %d %d\n", kEriClasses[c].name, B->block[c], B->chunk[c], B->bps[c]);
             fclose(f);
