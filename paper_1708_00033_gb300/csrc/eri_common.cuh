@@ -399,11 +399,11 @@ __device__ __forceinline__ void warp_bitonic_sort(unsigned* k, int n, int lane32
                 }                                                                                            \
                 if constexpr (SOA) {                                                                         \
                     const KetSoa<real> kv{(const real*)a.kt + k, a.ktB + k, a.kstride};                      \
-                    nprimq += QFN<real, GK>(hb, hk, kv, prims, bt, P, a.N, f, Jt, Kt, nullptr, pt, lane,     \
+                    nprimq += QFN<real, GK>(hb, hk, kv, prims, bt, P, a.N, f, Jt, Kt, pt, lane,              \
                                             live);                                                           \
                 } else {                                                                                     \
                     const KetAos<real> kv{prims + hk.prim0};                                                 \
-                    nprimq += QFN<real, GK>(hb, hk, kv, prims, bt, P, a.N, f, Jt, Kt, nullptr, pt, lane,     \
+                    nprimq += QFN<real, GK>(hb, hk, kv, prims, bt, P, a.N, f, Jt, Kt, pt, lane,              \
                                             live);                                                           \
                 }                                                                                            \
             }                                                                                                \

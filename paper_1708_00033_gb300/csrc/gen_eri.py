@@ -667,7 +667,7 @@ def gen_class(X, Y, method="os"):
     out.append(f"template <typename real, int G, typename KV>")
     out.append(f"__device__ __forceinline__ int {qname}(const PairHdr& hb, const PairHdr& hk, const KV& kv,"
                f" const PrimPair<real>* __restrict__ prims, const real* __restrict__ boys_tab,")
-    out.append(f"    const real* __restrict__ Pd, int N, real fscale, double* __restrict__ Jt, double* __restrict__ Kt, double* qout,")
+    out.append(f"    const real* __restrict__ Pd, int N, real fscale, double* __restrict__ Jt, double* __restrict__ Kt,")
     out.append(f"    float ptau, int lane, bool valid)")
     out.append("{")
     out.append("    // surviving primitive quartets form a staircase (pairs sorted by bound): bra primitive ib pairs")
@@ -715,12 +715,6 @@ def gen_class(X, Y, method="os"):
         tail.append("const real CDx = pair_ab<real>(hk.ABx, hk.ABfx), CDy = pair_ab<real>(hk.ABy, hk.ABfy), "
                     "CDz = pair_ab<real>(hk.ABz, hk.ABfz);")
     tail += hrr
-    tail.append("if (qout) {")
-    if X == Y:
-        tail += ["    " + l for l in gen_schwarz(la, lb, xname)]
-        tail.append("    *qout = qmax;")
-    tail.append("    return;")
-    tail.append("}")
     tail.append("if (total == 0) return;  // every primitive quartet screened: nothing to digest")
     tail.append("const int bA = hb.bfA, bB = hb.bfB, bC = hk.bfA, bD = hk.bfB;")
     tail.append("const real fj = real(4) * fscale, fk = real(2) * fscale;")

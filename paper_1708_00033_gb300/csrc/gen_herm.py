@@ -398,13 +398,13 @@ def gen_warp(name, la, lb, lc, ld):
     o.append(f"struct HermWarp_{name} {{")
     nrp = len(hs) | 1
     o.append(f"    static constexpr int NR = {len(hs)}, NRP = {nrp}, NBS = {len(B)}, NKS = {len(K)}, NACC = {len(acc)},"
-             f" NSLOT = {nslot}, NBI = {len(BI)}, NKI = {len(KI)}, NE = {len(es)}, NF = {len(fs)};")
+             f" NSLOT = {nslot}, NKI = {len(KI)}, NE = {len(es)}, NF = {len(fs)};")
     o.append(f"    static constexpr int LA = {la}, LB = {lb}, LC = {lc}, LD = {ld};")
-    # quartets per group: enough (quartet, ket item) columns for the lanes; one where L >= 7 needs the shared memory
+    # quartets per group: about a warp's worth of (quartet, ket item) columns, or more where one quartet exceeds it (11
+    # items: 33 columns, the last of them in a round of its own); one where L >= 7 needs the shared memory
     ng = 1 if L >= 7 else {1: 8, 4: 8, 11: 3, 15: 2, 35: 2}[len(KI)]
     o.append(f"    static constexpr int NQ = {ng};")
     o.append("    static __device__ __forceinline__ const unsigned short* slots() { return kHermSlot_%s; }" % name)
-    o.append("    static __device__ __forceinline__ const unsigned short* item_table() { return kHermItem_%s; }" % name)
     o.append("    // one primitive quartet: R[0..NR), scalings sc[0..NBS + NKS)")
     o.append("    static __device__ __forceinline__ void prim(const HermPair& bp, const HermPair& kp, const double2* __restrict__ etab,"
              " int ntype, const double* __restrict__ boys_tab, double live, double* __restrict__ R, double* __restrict__ sc)")
