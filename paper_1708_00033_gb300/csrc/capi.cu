@@ -441,7 +441,7 @@ static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* b
     KCHK(launch_class_count(npairs, S->pair_class.as<int>(), cnt_dev, st));
     unsigned long long cnt_all[kNumPairClasses];
     HF_CUDA(cudaMemcpyAsync(cnt_all, cnt_dev, sizeof(cnt_all), cudaMemcpyDeviceToHost, st));
-    HF_CUDA(cudaStreamSynchronize(st));  // host sync 1 of 2: class sizes
+    HF_CUDA(cudaStreamSynchronize(st));  // host sync: class sizes
 
     // ------------------------------------------------------ schedule arena
     size_t npad[kNumPairClasses], seg[kNumPairClasses + 1], base_all[kNumPairClasses + 1];
@@ -550,7 +550,7 @@ static int system_setup(hf_system* S, const hf_geometry* geom, const hf_basis* b
     HF_CUDA(cudaMemcpyAsync(enn_dev + 1, qbits_dev, sizeof(double), cudaMemcpyDeviceToDevice, st));
     unsigned char rbh[512];
     HF_CUDA(cudaMemcpyAsync(rbh, rb.p, 512, cudaMemcpyDeviceToHost, st));
-    HF_CUDA(cudaStreamSynchronize(st));  // host sync 2 of 2: significant counts, quartet totals, E_nn
+    HF_CUDA(cudaStreamSynchronize(st));  // host sync: significant counts, quartet totals, E_nn
     const unsigned* nsig_h = (const unsigned*)rbh;
     const long long* totals_h = (const long long*)(rbh + 32);
     memcpy(&S->E_nn, rbh + 32 + 8 * 2 * kNumClasses, sizeof(double));

@@ -30,8 +30,8 @@ struct PairHdr {
     float ABfx, ABfy, ABfz;  // A - B in FP32 (the FP32 kernels' horizontal step uses no FP64 instruction)
 };
 
-// Primitive-pair record of the Hermite-accumulator kernels: P, K (a + b)^-W with the prefactor K of PrimPair
-// and W = l_A + l_B, u = 2b, v = 2p, and the type of p in the exponent table.  Four 16-byte loads.
+// Primitive-pair record of the Hermite-accumulator kernels: P, K (2p)^-W with the prefactor K of PrimPair,
+// p = a + b and W = l_A + l_B, u = 2b, v = 2p, and the type of p in the exponent table.  Four 16-byte loads.
 struct alignas(16) HermPair {
     double Px, Py, Pz;
     double K;

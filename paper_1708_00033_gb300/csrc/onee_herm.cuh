@@ -49,9 +49,10 @@ __device__ __forceinline__ void one_electron_pair(const OneEArgs& a, int pid, do
     const double* const cb = a.cn + a.prim0[h.B];
     const double AB[3] = {h.ABx, h.ABy, h.ABz};
     const double R2 = AB[0] * AB[0] + AB[1] * AB[1] + AB[2] * AB[2];
-    // primitive pairs whose Gaussian-product factor exp(-ab/(a+b) |AB|^2) is below exp(-60) ~ 9e-27 are skipped:
-    // with normalised coefficients below 1e3, 2 pi / p below 30, a total nuclear charge below 1e5 and polynomial
-    // factors below 1e6 their contribution to any element stays below 1e-12 of the 1e-11 parity tolerance
+    // primitive pairs whose Gaussian-product factor exp(-x), x = ab/(a+b) |AB|^2, is below exp(-60) ~ 9e-27 are
+    // skipped.  Functions and primitives are normalised, so with two contraction coefficients below 10 each, the
+    // components' polynomials ((4 x)^2 at most for two d functions, 6e4 here) and 1e6 for total charge times
+    // 2 sqrt(p), what is dropped from an element stays below 6e-14, a hundredth of the 1e-11 parity tolerance
     auto skipped = [&](double x, double y) { return x * y / (x + y) * R2 > 60.0; };
     double sa[(NAB + 31) / 32], ta[(NAB + 31) / 32];
 #pragma unroll
