@@ -37,7 +37,8 @@ DFMA_PEAK_GFLOPS = 152 * 2 * 2 * 2.070  # 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.
 # ncu capture of the default workload, with the SHA-256 of the sources that kernel is compiled from at that
 # time; the bench reports it only while those sources are unchanged (else the counters describe another
 # kernel and traffic is null).
-NCU_TRAFFIC = {"kernel": "k_herm_1110", "bytes_per_launch": None, "sources_sha256": None}
+NCU_TRAFFIC = {"kernel": "k_herm_1110", "bytes_per_launch": 113_864_448,
+               "sources_sha256": "74baec6058f4f2fd0a78d393d1363a9c6d79cb625b6d0acefaf0f322cee4e0cc"}
 TRAFFIC_SOURCES = ("paper_1708_00033_gb300/csrc/gen_eri.py", "paper_1708_00033_gb300/csrc/gen_herm.py",
                    "paper_1708_00033_gb300/csrc/eri_common.cuh", "paper_1708_00033_gb300/csrc/eri_herm.cuh",
                    "paper_1708_00033_gb300/csrc/hf_internal.h")
