@@ -392,14 +392,14 @@ int hf_batch_offsets(const hf_batch* batch, int64_t* off);
 int hf_fock_build_batch(hf_batch* batch, const double* P, double* F, double* E_elec, float* ms, int flags);
 
 /* Autotuner: for every class kernel, time each candidate (block size 64/128/
- * 256, chunk 32/128/256/512 quartets, 2/4/8 blocks per SM; kernels of one warp
- * per block: blocks per SM only) on the class's first quartets - as many as
- * take about 2e10 algorithmic operations, at most sample_quartets (0: 2e6) -
- * and keep the fastest; choices are read from and written to cache_path when
- * it is not NULL (a header line with the format and the device, then one
- * "class block chunk blocks_per_sm" line per class; a file with another header
- * is ignored and rewritten).  Re-captures the graph.  Errors: HF_E_INVALID,
- * HF_E_CUDA. */
+ * 256, chunk 256/512 and for small batches 32/128 quartets, 2/4/8 blocks per
+ * SM; kernels of one warp per block: blocks per SM only) on the class's first
+ * quartets - as many as take about 2e10 algorithmic operations, at most
+ * sample_quartets (0: 2e6) - and keep the fastest; choices are read from and
+ * written to cache_path when it is not NULL (a header line with the format and
+ * the device, then one "class block chunk blocks_per_sm" line per class; a file
+ * with another header is ignored and rewritten).  Re-captures the graph.
+ * Errors: HF_E_INVALID, HF_E_CUDA. */
 int hf_batch_tune(hf_batch* batch, const char* cache_path, int64_t sample_quartets);
 
 /* --------------------------------------------------------- learned guess */

@@ -47,3 +47,18 @@ def test_other_files_are_ignored(tmp_path, header):
     counts, before, after = _tuned(path)
     assert len(counts) == hf.NUM_CLASSES and after == before
     assert path.read_text().startswith("# hf_batch_tune format 2, recorded sm_103\n")
+
+
+def test_chunks_below_the_sorted_window_are_for_small_batches():
+    """Every class of this batch has 400,000 quartets, more than four windows per resident warp together."""
+    geom = inputs.batch_cluster(inputs.CONFIG_BATCH, 0, 1, 1)
+    with recorded() as (lib, ctx):
+        lib.rec_read_words(1, 400_000)
+        batch = hf.Batch(ctx, [geom], [inputs.synthetic_basis(geom)])
+        lib.rec_clear()
+        batch.tune()
+        counts = Counter(re.search(r"k_eri_batch_(\d{4})", w).group(1) for op, _, w in log(lib)
+                         if op == "launch" and "k_eri_batch" in w)
+        batch.close()
+    for name, n in counts.items():
+        assert n == 2 * (3 if sum(map(int, name)) > 4 else 3 * 2 * 3), name
